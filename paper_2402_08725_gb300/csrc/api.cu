@@ -227,12 +227,41 @@ struct Plan {
     bool profiling = false;
     int prof_count = 0;
     std::vector<cudaEvent_t> prof_ev;
+    // The prior branch: the starlet levels (and the point-source prior) read only the parameters
+    // and write their own buffers, so they run on this stream beside the chi^2 branch, between a
+    // fork at the start of the evaluation and a join before dL/dh (NULL: everything in order on
+    // the evaluation's stream).  A plan's evaluations are ordered by its owner's stream, which
+    // both events tie the branch to, so one stream per plan is enough.
+    cudaStream_t side = nullptr;
+    cudaEvent_t side_fork = nullptr, side_join = nullptr;
     DevArena arena;
     ~Plan() {
         if (graph) cudaGraphExecDestroy(graph);
         for (cudaEvent_t e : prof_ev) cudaEventDestroy(e);
+        if (side_fork) cudaEventDestroy(side_fork);
+        if (side_join) cudaEventDestroy(side_join);
+        if (side) cudaStreamDestroy(side);
     }
 };
+
+// The stream of the evaluation's prior branch, ordered after everything queued on `st` so far;
+// `st` itself when the plan has no branch (or the fork fails: the order is then kept).
+static cudaStream_t fork_prior(Plan *pl, cudaStream_t st) {
+    if (!pl->side) return st;
+    if (cudaEventRecord(pl->side_fork, st) != cudaSuccess ||
+        cudaStreamWaitEvent(pl->side, pl->side_fork, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return st;
+    }
+    return pl->side;
+}
+
+// Orders `st` after the branch.
+static void join_prior(Plan *pl, cudaStream_t branch, cudaStream_t st) {
+    if (branch == st) return;
+    cudaEventRecord(pl->side_join, branch);
+    cudaStreamWaitEvent(st, pl->side_join, 0);
+}
 
 struct sr_problem {
     sr_problem_desc desc{};
@@ -813,6 +842,11 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
             pl->grid_adj = std::min(pl->grid_adj, opt.grid_limit);
         }
     }
+    if (!plain && opt.grid_limit == 0) {  // (the form autotuner times its plans in order)
+        SR_CUDA(cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking));
+        SR_CUDA(cudaEventCreateWithFlags(&pl->side_fork, cudaEventDisableTiming));
+        SR_CUDA(cudaEventCreateWithFlags(&pl->side_join, cudaEventDisableTiming));
+    }
     return SR_OK;
 }
 
@@ -821,8 +855,13 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
                     const std::vector<const float *> *s_raw) {
     int n = 0;
     if (pl->kind == SR_PSF) {
-        n += launch_psf_eval(pl->d_fields, pl->h_fields[0], pl->d_chunks, pl->n_chunks, params, grad, pl->psf,
-                             pl->l1_part, pl->losses, pl->total, st);
+        const FieldDev &hf = pl->h_fields[0];
+        cudaStream_t prior = fork_prior(pl, st);
+        n += launch_psf_chi(pl->d_fields, hf, params, pl->psf, st);
+        n += launch_starlet(pl->d_fields, 1, hf.F, starlet_forms_single(hf.F, hf.J, hf.Wmap != nullptr), pl->d_chunks,
+                            pl->n_chunks, hf.J, params, pl->l1_part, prior);
+        join_prior(pl, prior, st);
+        n += launch_psf_finish(pl->d_fields, hf, params, grad, pl->psf, pl->l1_part, pl->losses, pl->total, st);
         return n;
     }
     if (pl->plain) {
@@ -831,6 +870,7 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
                                pl->l1_part, pl->losses, pl->total, st);
         return n;
     }
+    cudaStream_t prior = fork_prior(pl, st);  // launched after the chi^2 branch, whose chain is the longer one
     cudaMemsetAsync(pl->d_counters, 0, 4 * sizeof(int), st);
     cudaEvent_t *ev = nullptr;
     if (pl->profiling && !pl->prof_ev.empty()) {
@@ -867,7 +907,12 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
         ++n;
     }
     n += launch_starlet(pl->d_fields, pl->n_fields, pl->Fmax, pl->starlet_forms, pl->d_chunks, pl->n_chunks, pl->Jmax,
-                        params, pl->l1_part, st);
+                        params, pl->l1_part, prior);
+    if (pl->n_sh > 0)
+        n += launch_pts_prior(pl->d_sh, pl->d_fields, pl->n_sh, pl->sh_Fmax, pl->sh_Mmax, pl->sh_starlet_forms,
+                              pl->d_sh_chunks, pl->n_sh_chunks, pl->sh_Jmax, params, pl->abar, pl->pbar, pl->l1_pts,
+                              pl->pts_g, prior);
+    join_prior(pl, prior, st);
     if (pl->n_items > 0) {
         launch_hgrad(pl->d_fields, pl->d_chunks, pl->n_chunks, pl->gbuf, grad, params, st);
         ++n;
@@ -882,10 +927,6 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
     }
     for (size_t b = 0; b < pl->big_fields.size(); ++b)
         n += launch_big_hgrad(pl->h_fields[pl->big_fields[b]], pl->big_buf[b], grad, st);
-    if (pl->n_sh > 0)
-        n += launch_pts_prior(pl->d_sh, pl->d_fields, pl->n_sh, pl->sh_Fmax, pl->sh_Mmax, pl->sh_starlet_forms,
-                              pl->d_sh_chunks, pl->n_sh_chunks, pl->sh_Jmax, params, pl->abar, pl->pbar, pl->l1_pts,
-                              pl->pts_g, st);
     launch_finalize(pl->d_fields, pl->n_fields, pl->chi_part, pl->se_part, pl->l1_part, pl->ps_da, pl->ps_du, grad,
                     pl->losses, pl->total, st, pl->n_sh > 0 ? pl->d_sh : nullptr, pl->l1_pts, pl->pts_g, pl->hs);
     n += 2;

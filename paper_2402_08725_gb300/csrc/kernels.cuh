@@ -143,9 +143,12 @@ struct PsfBuffers {
     double *ab_part;    // [n_chunks][2]: dalpha, dbeta partials
     int n_dchunks;      // data-grid chunks per star
 };
-int launch_psf_eval(const FieldDev *fields, const FieldDev &host_field, const ChunkItem *chunks, int n_chunks,
-                    const float *params, float *grad, const PsfBuffers &pb, double *l1_part, double *losses,
-                    double *total, cudaStream_t st);
+// An evaluation: launch_psf_chi, the starlet prior on b (launch_starlet, in either order or beside
+// it), then launch_psf_finish.
+int launch_psf_chi(const FieldDev *fields, const FieldDev &host_field, const float *params, const PsfBuffers &pb,
+                   cudaStream_t st);
+int launch_psf_finish(const FieldDev *fields, const FieldDev &host_field, const float *params, float *grad,
+                      const PsfBuffers &pb, double *l1_part, double *losses, double *total, cudaStream_t st);
 
 // The narrow PSF s = Moffat(alpha, beta) + b of the parameters, into fields[0].psf_s.
 void launch_psf_model(const FieldDev *fields, int F, const float *params, cudaStream_t st);

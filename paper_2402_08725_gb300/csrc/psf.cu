@@ -258,9 +258,9 @@ void launch_psf_model(const FieldDev *fields, int F, const float *params, cudaSt
     psf_build_s_kernel<<<(F * F + 255) / 256, 256, 0, st>>>(fields, params);
 }
 
-int launch_psf_eval(const FieldDev *fields, const FieldDev &hf, const ChunkItem *chunks, int n_chunks,
-                    const float *params, float *grad, const PsfBuffers &pb, double *l1_part, double *losses,
-                    double *total, cudaStream_t st) {
+// The chi^2 part: residuals, the stars' partial sums and their gradients with respect to s.
+int launch_psf_chi(const FieldDev *fields, const FieldDev &hf, const float *params, const PsfBuffers &pb,
+                   cudaStream_t st) {
     const int F = hf.F;
     const long long nst = (long long)hf.E * F * F;
     const int gF = (F * F + 255) / 256;
@@ -272,12 +272,17 @@ int launch_psf_eval(const FieldDev *fields, const FieldDev &hf, const ChunkItem 
                                                                  pb.n_dchunks); ++n;
     psf_adj_col_kernel<<<gS, 256, 0, st>>>(fields, params, pb.ebuf); ++n;
     psf_adj_row_kernel<<<gS, 256, 0, st>>>(fields, params); ++n;
-    const int forms = starlet_forms_single(hf.F, hf.J, hf.Wmap != nullptr);
-    n += launch_starlet(fields, 1, hf.F, forms, chunks, n_chunks, hf.J, params, l1_part, st);
-    psf_reduce_kernel<<<gF, 256, 0, st>>>(fields, params, grad, pb.ab_part); ++n;
-    psf_finalize_kernel<<<1, 256, 0, st>>>(fields, params, grad, pb.star_part, pb.n_dchunks, pb.ab_part, gF,
-                                           l1_part, losses, total); ++n;
     return n;
+}
+
+// The sums over the stars, joined with the prior (starlet.cu) on b.
+int launch_psf_finish(const FieldDev *fields, const FieldDev &hf, const float *params, float *grad,
+                      const PsfBuffers &pb, double *l1_part, double *losses, double *total, cudaStream_t st) {
+    const int gF = (hf.F * hf.F + 255) / 256;
+    psf_reduce_kernel<<<gF, 256, 0, st>>>(fields, params, grad, pb.ab_part);
+    psf_finalize_kernel<<<1, 256, 0, st>>>(fields, params, grad, pb.star_part, pb.n_dchunks, pb.ab_part, gF,
+                                           l1_part, losses, total);
+    return 2;
 }
 
 }  // namespace sr
