@@ -16,18 +16,21 @@
 //
 // Work per batch of B realisations (all resident in L2):
 //   noise_draw_kernel      x[b]  = z / sigma_eff^                     (one Philox block a thread)
-//   noise_corr_kernel      y[b]  = S_1^T x[b]                          (FP32, 2 F^2 K^2 flop each)
+//   noise_corr_kernel      y[b]  = S_1^T x[b]                          (FP32, 2 F^2 K^2 flop each), or
+//   noise_fft_kernel       the same by transforms (noise_fft.cu), where that is cheaper
 //   noise_row_kernel       t[b]  = row pass of level j on c_j[b]
-//   noise_col_stats_kernel c_{j+1}[b] = column pass; w = c_j - c_{j+1}; FP64 sum and sum of
-//                          squares of w over the batch, in a fixed order, into per-segment
-//                          accumulators
+//   noise_col_stats_kernel c_{j+1}[b] = column pass; w = c_j - c_{j+1}; sum and sum of squares of
+//                          w over the batch, in a fixed order, into per-segment FP64 accumulators
 // and at the end noise_map_kernel / noise_scale_kernel reduce the segments in a fixed order.
-// The correlation dominates: it is bound by FP32 FMA issue.
+// The direct correlation is bound by FP32 FMA issue (5000 realisations at F = 128, K = 64: 11.7 ms);
+// with the transforms (0.78 ms) the column passes are the largest part.
 #include <algorithm>
 #include <cmath>
 #include <vector>
 
 #include "common.cuh"
+#include "ffsum.cuh"
+#include "noise.cuh"
 
 namespace sr {
 namespace {
@@ -55,15 +58,21 @@ __device__ __forceinline__ void philox4x64_10(uint64_t &c0, uint64_t &c1, uint64
 
 __device__ __forceinline__ float uniform24(uint64_t w) { return (float)((w >> 40) + 1) * 0x1p-24f; }
 
-// x[b][u] = z(seed, (r0 + b) F^2 + u) * isig[u] for the n = B F^2 numbers of the batch.
+// x[b][u] = z(seed, (r0 + b) F^2 + u) * isig[u] for the n = B F^2 numbers of the batch.  The batch
+// starts at pixel 0 of its first realisation, so the pixel of number n0 + i is i mod F^2, in 32 bits
+// (Int) unless one realisation alone is larger than that: a 64-bit remainder per number cost as much
+// as the generator (5000 realisations at F = 128: 0.53 ms before, 0.43 ms with this).
+template <typename Int>
 __global__ void __launch_bounds__(256) noise_draw_kernel(const float *__restrict__ isig, int F, uint64_t seed,
                                                          long long r0, int B, float *__restrict__ x) {
-    const long long FF = (long long)F * F;
-    const long long n0 = r0 * FF, n1 = n0 + (long long)B * FF;
-    const long long blk0 = n0 >> 2, blk1 = (n1 - 1) >> 2;
-    for (long long blk = blk0 + blockIdx.x * (long long)blockDim.x + threadIdx.x; blk <= blk1;
-         blk += (long long)gridDim.x * blockDim.x) {
-        uint64_t c0 = (uint64_t)blk, c1 = 0, c2 = 0, c3 = 0;
+    const Int FF = (Int)F * F;
+    const long long n0 = r0 * FF;
+    const Int total = B * FF;
+    const int lead = (int)(n0 & 3);  // the first block's numbers before the batch
+    const long long blk0 = n0 >> 2;
+    const Int nblk = (lead + total + 3) >> 2;
+    for (Int k = blockIdx.x * blockDim.x + threadIdx.x; k < nblk; k += gridDim.x * blockDim.x) {
+        uint64_t c0 = (uint64_t)(blk0 + k), c1 = 0, c2 = 0, c3 = 0;
         philox4x64_10(c0, c1, c2, c3, seed, 0);
         float z[4];
         {
@@ -80,12 +89,14 @@ __global__ void __launch_bounds__(256) noise_draw_kernel(const float *__restrict
             z[2] = r * c;
             z[3] = r * s;
         }
+        const Int i0 = 4 * k - lead;
+        Int u = (i0 < 0 ? 0 : i0) % FF;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const long long n = 4 * blk + e;
-            if (n < n0 || n >= n1) continue;
-            const long long u = n % FF;
-            x[n - n0] = z[e] * isig[u];
+            const Int i = i0 + e;
+            if (i < 0 || i >= total) continue;
+            x[i] = z[e] * isig[u];
+            if (++u == FF) u = 0;
         }
     }
 }
@@ -220,7 +231,7 @@ __global__ void __launch_bounds__(256) noise_row_kernel(const float *__restrict_
 // Column pass of level j for the realisations of segment blockIdx.y, pixel u per thread:
 // c_{j+1} = column filter of t, w = c_j - c_{j+1} (c updated in place: only this thread reads or
 // writes c[b][u]); the segment's sums of w and w^2, taken over b in increasing order (groups of
-// four in FP32, the groups in FP64), are added to acc1/acc2[seg][j][u].
+// four in FP32, the groups as compensated pairs), are added to acc1/acc2[seg][j][u].
 __global__ void __launch_bounds__(256) noise_col_stats_kernel(float *__restrict__ c, const float *__restrict__ t,
                                                               int F, int step, int B, int S, int J1, int j,
                                                               double *__restrict__ acc1, double *__restrict__ acc2) {
@@ -232,7 +243,7 @@ __global__ void __launch_bounds__(256) noise_col_stats_kernel(float *__restrict_
     const int yy = (int)(u / F), xx = (int)(u - (long long)yy * F);
     const long long o_m2 = (long long)reflect(yy - 2 * step, F) * F + xx, o_p2 = (long long)reflect(yy + 2 * step, F) * F + xx;
     const long long o_m1 = (long long)reflect(yy - step, F) * F + xx, o_p1 = (long long)reflect(yy + step, F) * F + xx;
-    double s1 = 0.0, s2 = 0.0;
+    FSum s1 = fsum_zero(), s2 = fsum_zero();
     int b = b0;
     for (; b + 4 <= b1; b += 4) {  // four realisations' loads issued before their arithmetic
         float tv[4][5], cv[4];
@@ -246,8 +257,9 @@ __global__ void __launch_bounds__(256) noise_col_stats_kernel(float *__restrict_
             tv[k][4] = tb[o_p2];
             cv[k] = c[(b + k) * FF + u];
         }
-        // the four realisations summed in FP32 (in order), then added to the FP64 sums: a quarter
-        // of the FP64 operations, which run at a small fraction of the FP32 rate
+        // the four realisations summed in FP32 (in order), then added to the segment's sums as
+        // compensated FP32 pairs (48 significand bits; FP64 additions run at 2 a clock per SM and
+        // took a fifth of the column passes: 2.4 -> 1.95 ms per 5000 realisations at F = 128, J = 4)
         float q1 = 0.f, q2 = 0.f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -257,8 +269,8 @@ __global__ void __launch_bounds__(256) noise_col_stats_kernel(float *__restrict_
             q1 += w;
             q2 = fmaf(w, w, q2);
         }
-        s1 += (double)q1;
-        s2 += (double)q2;
+        s1 = fsum_add(s1, q1);
+        s2 = fsum_add(s2, q2);
     }
     for (; b < b1; ++b) {
         const float *tb = t + b * FF;
@@ -266,12 +278,13 @@ __global__ void __launch_bounds__(256) noise_col_stats_kernel(float *__restrict_
         float *cb = c + b * FF + u;
         const float w = *cb - cn;
         *cb = cn;
-        s1 += (double)w;
-        s2 += (double)w * (double)w;
+        s1 = fsum_add(s1, w);
+        const float w2 = w * w;
+        s2 = fsum_add(s2, FSum{w2, fmaf(w, w, -w2)});
     }
     const long long k = ((long long)seg * J1 + j) * FF + u;
-    acc1[k] += s1;
-    acc2[k] += s2;
+    acc1[k] += fsum_value(s1);
+    acc2[k] += fsum_value(s2);
 }
 
 // W_map[j][u] = sample std (n - 1) of w_{j+1}[u] over the n realisations (segments summed in order).
@@ -289,17 +302,22 @@ __global__ void __launch_bounds__(256) noise_map_kernel(const double *__restrict
     W_map[k] = (float)sqrt(var > 0.0 ? var : 0.0);
 }
 
-// W_scale[j] = sample std (n F^2 - 1) of every coefficient of plane j: one block per plane, a
-// strided per-thread sum then a fixed-shape tree.
-constexpr int kScaleThreads = 256;
+// W_scale[j] = sample std (n F^2 - 1) of every coefficient of plane j, in two fixed-shape steps:
+// block (b, j) sums its share of the plane's pixels over the segments, and the last block of the
+// plane to finish (counted in done[j], zero before the launch) adds the blocks' partials.  (One block per plane took 0.30 ms at F = 128: its loads are a single chain
+// of 64 x 16 per thread.)
+constexpr int kScaleThreads = 256, kScaleBlocks = 64;
 __global__ void __launch_bounds__(kScaleThreads) noise_scale_kernel(const double *__restrict__ acc1,
                                                                     const double *__restrict__ acc2, long long FF,
-                                                                    int J1, int S, int n, float *__restrict__ W) {
+                                                                    int J1, int S, int n, double2 *part, int *done,
+                                                                    float *__restrict__ W) {
     __shared__ double r1[kScaleThreads], r2[kScaleThreads];
-    const int j = blockIdx.x;
+    __shared__ bool s_last;
+    const int j = blockIdx.y;
     const long long per_seg = FF * J1;
     double t1 = 0.0, t2 = 0.0;
-    for (long long u = threadIdx.x; u < FF; u += kScaleThreads)
+    for (long long u = blockIdx.x * (long long)kScaleThreads + threadIdx.x; u < FF; u += kScaleBlocks * kScaleThreads)
+#pragma unroll 4
         for (int s = 0; s < S; ++s) {
             t1 += acc1[s * per_seg + j * FF + u];
             t2 += acc2[s * per_seg + j * FF + u];
@@ -315,49 +333,176 @@ __global__ void __launch_bounds__(kScaleThreads) noise_scale_kernel(const double
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        const double m = (double)n * (double)FF, mean = r1[0] / m, var = (r2[0] - m * mean * mean) / (m - 1.0);
+        part[j * kScaleBlocks + blockIdx.x] = make_double2(r1[0], r2[0]);
+        __threadfence();
+        s_last = atomicAdd(&done[j], 1) == kScaleBlocks - 1;
+    }
+    __syncthreads();
+    if (!s_last || threadIdx.x >= 32) return;
+    __threadfence();
+    t1 = t2 = 0.0;
+    for (int b = threadIdx.x; b < kScaleBlocks; b += 32) {
+        const double2 v = __ldcg(&part[j * kScaleBlocks + b]);
+        t1 += v.x;
+        t2 += v.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        t1 += __shfl_down_sync(0xffffffffu, t1, o);
+        t2 += __shfl_down_sync(0xffffffffu, t2, o);
+    }
+    if (threadIdx.x == 0) {
+        const double m = (double)n * (double)FF, mean = t1 / m, var = (t2 - m * mean * mean) / (m - 1.0);
         W[j] = (float)sqrt(var > 0.0 ? var : 0.0);
     }
 }
 
-// 1/sigma_eff on the fine grid; flags (bit 0) a NaN or non-positive sigma and (bit 1) a
-// non-finite PSF value.
-__global__ void __launch_bounds__(256) noise_isig_kernel(const float *__restrict__ sigma, const float *__restrict__ s1,
-                                                         int N, int f, int E, int K, float *__restrict__ isig,
-                                                         int *__restrict__ flag) {
-    const int F = f * N;
-    const long long FF = (long long)F * F, KK = (long long)K * K;
-    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < FF || u < KK;
-         u += (long long)gridDim.x * blockDim.x) {
-        if (u < KK && !isfinite(s1[u])) atomicOr(flag, 2);
-        if (u >= FF) continue;
-        const int yy = (int)(u / F), xx = (int)(u % F);
-        const long long p = (long long)(yy / f) * N + xx / f;
+// 1/sg^2 in FP64: an FP32 reciprocal and one Newton step (relative error below 1e-13; a division
+// is about three times the FP64 operations, which run at 2 a clock per SM), or the division itself
+// where sg^2 would leave the normal FP32 range.
+__device__ __forceinline__ double inv_square(float sg) {
+    const double s2 = (double)sg * (double)sg;
+    if (!(sg > 1e-15f && sg < 1e15f)) return 1.0 / s2;
+    const double r = (double)(1.f / (sg * sg));
+    return fma(r, fma(-s2, r, 1.0), r);
+}
+
+// The set-up of a call, one launch:
+// blocks [0, n_isig): 1/sigma_eff on the fine grid; flags (bit 0) a NaN or non-positive sigma and
+//   (bit 1) a non-finite PSF value.  A block takes 32 data pixels (lanes) and deals the epochs over
+//   its 8 warps (epoch i to warp i mod 8, the warps' sums added in order), so that the epochs' loads
+//   are in flight together; one thread per fine pixel walking every epoch took 0.25 ms at E = 300,
+//   N = 64.
+// blocks n_isig + kx, kx < spec.L: column kx of the transform form's kernel spectrum (noise_spectrum).
+constexpr int kIsigWarps = 8;
+
+__device__ void noise_isig(const float *__restrict__ sigma, const float *__restrict__ s1, int N, int f, int E, int K,
+                           int n_blocks, float *__restrict__ isig, int *__restrict__ flag,
+                           double (*part)[32]) {
+    const int F = f * N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long NN = (long long)N * N, KK = (long long)K * K;
+    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < KK; u += (long long)n_blocks * blockDim.x)
+        if (!isfinite(s1[u])) atomicOr(flag, 2);
+    for (long long p0 = blockIdx.x * 32LL; p0 < NN; p0 += n_blocks * 32LL) {
+        const long long p = p0 + lane;
         double iv = 0.0;
-        for (int i = 0; i < E; ++i) {
-            const float sg = sigma[(long long)i * N * N + p];
-            if (isnan(sg) || sg <= 0.f) atomicOr(flag, 1);
-            else if (isfinite(sg)) iv += 1.0 / ((double)sg * (double)sg);
+        bool bad = false;
+        if (p < NN) {
+#pragma unroll 4
+            for (int i = warp; i < E; i += kIsigWarps) {
+                const float sg = __ldg(sigma + i * NN + p);
+                if (isnan(sg) || sg <= 0.f) bad = true;
+                else if (isfinite(sg)) iv += inv_square(sg);
+            }
         }
-        isig[u] = (float)sqrt(iv);
+        if (bad) atomicOr(flag, 1);
+        part[warp][lane] = iv;
+        __syncthreads();
+        if (warp == 0 && p < NN) {
+            double t = 0.0;
+            for (int w = 0; w < kIsigWarps; ++w) t += part[w][lane];
+            const float v = (float)sqrt(t);
+            const int py = (int)(p / N), px = (int)(p - (long long)py * N);
+            for (int ay = 0; ay < f; ++ay)
+                for (int ax = 0; ax < f; ++ax) isig[(long long)(f * py + ay) * F + f * px + ax] = v;
+        }
+        __syncthreads();
     }
 }
 
-struct DevBufs {
-    std::vector<void *> ptrs;
-    ~DevBufs() {
-        for (void *p : ptrs) cudaFree(p);
+// Column kx of conj(Shat) / L^2 = L^-2 sum_{q,t} s[q][t] exp(2 pi i (ky (q - sh) + kx (t - sh)) / L),
+// summed over t, then over q, in FP64 and rounded once, at [position of ky][position of kx] of the
+// transforms' digit-transposed order (position R2 (k mod R1) + k / R1); kx = 0 also writes the
+// twiddles exp(-2 pi i j / L).
+constexpr int kSpecMax = 256;
+__device__ void noise_spectrum(const float *__restrict__ s, int K, int kx, const NoiseSpec &sp, double2 *w, double2 *R) {
+    const int L = sp.L, R2 = L / sp.R1;
+    for (int j = threadIdx.x; j < L; j += blockDim.x) {
+        double si, co;
+        sincospi(2.0 * (double)j / (double)L, &si, &co);
+        w[j] = make_double2(co, si);
+        if (kx == 0) sp.tw[j] = make_float2((float)co, (float)-si);
     }
-    template <class T> sr_status alloc(T **p, size_t count) {
+    __syncthreads();
+    for (int q = threadIdx.x; q < K; q += blockDim.x) {
+        double a = 0.0, b = 0.0;
+        int j = (int)((long long)kx * (L - sp.sh) % L);
+        for (int t = 0; t < K; ++t) {
+            const double v = (double)__ldg(s + (long long)q * K + t);
+            a += v * w[j].x;
+            b += v * w[j].y;
+            j += kx;
+            if (j >= L) j -= L;
+        }
+        R[q] = make_double2(a, b);
+    }
+    __syncthreads();
+    const double scale = 1.0 / ((double)L * (double)L);
+    const int pc = R2 * (kx % sp.R1) + kx / sp.R1;
+    for (int ky = threadIdx.x; ky < L; ky += blockDim.x) {
+        double a = 0.0, b = 0.0;
+        int j = (int)((long long)ky * (L - sp.sh) % L);
+        for (int q = 0; q < K; ++q) {
+            a += R[q].x * w[j].x - R[q].y * w[j].y;
+            b += R[q].x * w[j].y + R[q].y * w[j].x;
+            j += ky;
+            if (j >= L) j -= L;
+        }
+        sp.S[(long long)(R2 * (ky % sp.R1) + ky / sp.R1) * L + pc] = make_float2((float)(a * scale), (float)(b * scale));
+    }
+}
+
+__global__ void __launch_bounds__(32 * kIsigWarps)
+noise_setup_kernel(const float *__restrict__ sigma, const float *__restrict__ s1, int N, int f, int E, int K,
+                   int n_isig, float *__restrict__ isig, int *__restrict__ flag, NoiseSpec spec) {
+    __shared__ double2 w[kSpecMax], R[kSpecMax];
+    if ((int)blockIdx.x < n_isig)
+        noise_isig(sigma, s1, N, f, E, K, n_isig, isig, flag, reinterpret_cast<double (*)[32]>(w));
+    else
+        noise_spectrum(s1, K, blockIdx.x - n_isig, spec, w, R);
+}
+
+// Whether S_1^T runs as transforms (noise_fft.cu) rather than as the direct correlation, by cost per
+// realisation: the multiply-adds of the direct form (its whole 32 x 128 tiles, kernel rows padded to
+// 4) against the n^2 L^2 points of the transforms.  Measured per 1000 realisations (direct / transforms,
+// ms): equal at about 75 multiply-adds per point (F = 64, K = 5: 0.041 / 0.039 at 63; F = 144, K = 5:
+// 0.193 / 0.203 at 64; F = 90, K = 7: 0.068 / 0.076 at 75; F = 128, K = 9: 0.139 / 0.139 at 85); beyond,
+// F = 128, K = 15: 0.214 / 0.141, K = 64: 2.41 / 0.174; F = 200, K = 64 (2 x 2 tiles): 8.2 / 0.78.
+constexpr double kDirectPerPoint = 75.0;
+bool noise_uses_fft(int F, int K, int optin, NoiseFft *plan) {
+    if (!noise_fft_plan(F, K, optin, plan)) return false;
+    const double tiles = (double)((F + kCorrTX - 1) / kCorrTX) * ((F + kCorrTY - 1) / kCorrTY);
+    const double direct = tiles * kCorrTX * kCorrTY * K * ((K + 3) & ~3);
+    return direct > kDirectPerPoint * (double)plan->n * plan->n * plan->L * plan->L;
+}
+
+// The call's workspace in one allocation: blocks are reserved, then placed (each allocation and its
+// release cost about 50 us of host time, eleven of them a quarter of a call).
+struct Workspace {
+    struct Block {
+        void **p;
+        size_t off;
+    };
+    std::vector<Block> blocks;
+    size_t bytes = 0;
+    void *base = nullptr;
+    ~Workspace() {
+        if (base) cudaFree(base);
+    }
+    template <class T> void reserve(T **p, size_t count) {
         *p = nullptr;
-        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), count * sizeof(T) + 16);
+        blocks.push_back({reinterpret_cast<void **>(p), bytes});
+        bytes += (count * sizeof(T) + 255) / 256 * 256;
+    }
+    sr_status place() {
+        const cudaError_t e = cudaMalloc(&base, bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            set_error("sr_noise_weights: cudaMalloc of %zu bytes failed: %s", count * sizeof(T),
-                      cudaGetErrorString(e));
+            base = nullptr;
+            set_error("sr_noise_weights: cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
             return SR_ERR_OOM;
         }
-        ptrs.push_back(*p);
+        for (const Block &b : blocks) *b.p = static_cast<char *>(base) + b.off;
         return SR_OK;
     }
 };
@@ -407,6 +552,9 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
         set_error("sr_noise_weights: PSF size K = %d needs more shared memory than a block has", K);
         return SR_ERR_UNSUPPORTED;
     }
+    // the transform form of the correlation where it is the cheaper one
+    NoiseFft fft;
+    const bool use_fft = noise_uses_fft(F, K, optin, &fft);
     const size_t corr_smem = corr_smem_bytes(KP, KC);
     SR_CUDA(cudaFuncSetAttribute(noise_corr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)corr_smem));
     int occ = 0;
@@ -416,27 +564,47 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
     // batch: whole waves of correlation blocks, two F x F float buffers per realisation within 64 MB
     const long long FF = (long long)F * F;
     const int tiles_x = (F + kCorrTX - 1) / kCorrTX, tiles_y = (F + kCorrTY - 1) / kCorrTY;
-    const long long tiles = (long long)tiles_x * tiles_y, resident = (long long)occ * sms;
     const long long bmax = std::max(1LL, (64LL << 20) / (2 * 4 * FF));
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+
+    sr_status rc;
+    NoiseSpec spec;
+    long long tiles = (long long)tiles_x * tiles_y, resident = (long long)occ * sms;
+    if (use_fft) {
+        int blocks = 0;
+        if ((rc = noise_fft_prepare(fft, &blocks)) != SR_OK) return rc;
+        tiles = (long long)fft.n * fft.n;  // per pair of realisations
+        resident = 2LL * std::max(blocks, 1) * sms;
+    }
     long long B = std::max(1LL, (std::max(1LL, bmax * tiles / resident) * resident) / tiles);
     B = std::min({B, bmax, (long long)n_real, 65535LL});
+    if (use_fft && B < n_real && B > 1) B &= ~1LL;  // whole pairs of realisations
     // segments of the moment sums: enough threads in the column pass to fill the GPU
     const int S = (int)std::max(1LL, std::min({16LL, B, (sms * 2048LL + FF - 1) / FF}));
     const int J1 = J - 1;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-
-    DevBufs bufs;
+    Workspace ws;
     float *isig, *xbuf, *cbuf, *wsc;
+    double2 *scale_part;
     double *acc1, *acc2;
     int *flag;
-    sr_status rc;
-    if ((rc = bufs.alloc(&isig, FF)) || (rc = bufs.alloc(&xbuf, B * FF)) || (rc = bufs.alloc(&cbuf, B * FF)) ||
-        (rc = bufs.alloc(&acc1, (size_t)S * J1 * FF)) || (rc = bufs.alloc(&acc2, (size_t)S * J1 * FF)) ||
-        (rc = bufs.alloc(&wsc, J1)) || (rc = bufs.alloc(&flag, 1)))
-        return rc;
-    SR_CUDA(cudaMemsetAsync(acc1, 0, sizeof(double) * S * J1 * FF, st));
-    SR_CUDA(cudaMemsetAsync(acc2, 0, sizeof(double) * S * J1 * FF, st));
-    SR_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
+    ws.reserve(&acc1, (size_t)S * J1 * FF);
+    ws.reserve(&acc2, (size_t)S * J1 * FF);
+    ws.reserve(&flag, 1 + J1);
+    const size_t zeroed = ws.bytes;
+    ws.reserve(&isig, FF);
+    ws.reserve(&xbuf, B * FF);
+    ws.reserve(&cbuf, B * FF);
+    ws.reserve(&wsc, J1);
+    ws.reserve(&scale_part, (size_t)J1 * kScaleBlocks);
+    if (use_fft) {
+        ws.reserve(&spec.S, (size_t)fft.L * fft.L);
+        ws.reserve(&spec.tw, fft.L);
+        spec.L = fft.L;
+        spec.R1 = fft.R1;
+        spec.sh = fft.n == 1 ? K / 2 : 0;
+    }
+    if ((rc = ws.place()) != SR_OK) return rc;
+    SR_CUDA(cudaMemsetAsync(ws.base, 0, zeroed, st));  // the moments, the flag and the finishing counters
 
     cudaEvent_t ev[5] = {};
     const bool timed = timing != nullptr;
@@ -458,18 +626,27 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
         return ms;
     };
 
-    const int gs = (int)std::min<long long>((std::max(FF, (long long)K * K) + 255) / 256, sms * 8LL);
-    noise_isig_kernel<<<gs, 256, 0, st>>>(sigma_dev, s1_dev, N, f, E, K, isig, flag);
+    const int n_isig = (int)std::min<long long>(((long long)N * N + 31) / 32, sms * 8LL);
+    noise_setup_kernel<<<n_isig + spec.L, 32 * kIsigWarps, 0, st>>>(sigma_dev, s1_dev, N, f, E, K, n_isig, isig, flag,
+                                                                    spec);
     ++launches;
     for (long long r0 = 0; r0 < n_real; r0 += B) {
         const int Bb = (int)std::min(B, (long long)n_real - r0);
         if (timed) cudaEventRecord(ev[0], st);
         const long long nblk = ((r0 + Bb) * FF - 1) / 4 - (r0 * FF) / 4 + 1;
-        noise_draw_kernel<<<(int)std::min<long long>((nblk + 255) / 256, sms * 16LL), 256, 0, st>>>(
-            isig, F, seed, r0, Bb, xbuf);
+        const int gd = (int)std::min<long long>((nblk + 255) / 256, sms * 16LL);
+        if (Bb * FF < (1LL << 30)) noise_draw_kernel<int><<<gd, 256, 0, st>>>(isig, F, seed, r0, Bb, xbuf);
+        else noise_draw_kernel<long long><<<gd, 256, 0, st>>>(isig, F, seed, r0, Bb, xbuf);
         if (timed) cudaEventRecord(ev[1], st);
-        noise_corr_kernel<<<dim3(tiles_x, tiles_y, Bb), kCorrThreads, corr_smem, st>>>(xbuf, s1_dev, F, K, KP, KC,
-                                                                                       cbuf);
+        if (use_fft) {
+            if ((rc = launch_noise_fft(fft, xbuf, spec.S, spec.tw, F, K, Bb, sms, cbuf, st)) != SR_OK) {
+                destroy_events();
+                return rc;
+            }
+        } else {
+            noise_corr_kernel<<<dim3(tiles_x, tiles_y, Bb), kCorrThreads, corr_smem, st>>>(xbuf, s1_dev, F, K, KP, KC,
+                                                                                           cbuf);
+        }
         if (timed) cudaEventRecord(ev[2], st);
         const long long total = Bb * FF;
         const int Sb = std::min(S, Bb);
@@ -498,7 +675,8 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
         noise_map_kernel<<<(unsigned)((per + 255) / 256), 256, 0, st>>>(acc1, acc2, per, S, n_real, W_map_dev);
         ++launches;
     }
-    noise_scale_kernel<<<J1, kScaleThreads, 0, st>>>(acc1, acc2, FF, J1, S, n_real, wsc);
+    noise_scale_kernel<<<dim3(kScaleBlocks, J1), kScaleThreads, 0, st>>>(acc1, acc2, FF, J1, S, n_real, scale_part,
+                                                                           flag + 1, wsc);
     ++launches;
     if (timed) cudaEventRecord(ev[4], st);
     cudaError_t e = cudaGetLastError();
