@@ -439,8 +439,18 @@ static void fill_field_common(FieldDev &fd, sr_problem *p) {
     fd.Wmap = p->wmap_on ? p->wmap_dev : nullptr;
 }
 
-// Epochs per work item of the frequency-domain form (one accumulator per item).
-
+// Rows of the direct form's output tiles (64 columns wide): 64, or 32 or 16 for a field whose
+// (epoch, tile) items would not give every SM one.  A shorter tile stages more halo per output (Tk - 1
+// rows each) but runs more phases side by side in the block, so a field that leaves SMs idle gains
+// from it: 24 rotated epochs of 64 x 64 at Tk = 33, forward + adjoint kernel 357 us with 24 tiles of
+// 64 rows, 146 us with 96 of 16.  By the field's own shape, so that its sums do not depend on its
+// batch-mates.
+static int tile_rows(const sr_problem_desc &d, int n_sms) {
+    const long long across = (d.data_n + 63) / 64;
+    for (int rows : {64, 32})
+        if (d.n_epochs * across * ((d.data_n + rows - 1) / rows) >= n_sms) return rows;
+    return 16;
+}
 // Phase groups of a tile: the most phases at once that fit in the block's threads and in
 // shared memory (one group always).
 static int choose_pg(int nph, TileItem t, int Tk) {
@@ -630,13 +640,14 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
             }
             const int nph = fd.f * fd.f;
             std::vector<TileItem> tiles;
-            for (int y0 = 0; y0 < fd.N; y0 += 64)
+            const int rows = tile_rows(p->desc, g_num_sms);
+            for (int y0 = 0; y0 < fd.N; y0 += rows)
                 for (int x0 = 0; x0 < fd.N; x0 += 64) {
                     TileItem t{};
                     t.field = i;
                     t.y0 = (short)y0;
                     t.x0 = (short)x0;
-                    t.h = (short)std::min(64, fd.N - y0);
+                    t.h = (short)std::min(rows, fd.N - y0);
                     t.w = (short)(((std::min(64, fd.N - x0)) + kR - 1) / kR * kR);
                     t.pg = choose_pg(nph, t, fd.Tk);
                     tiles.push_back(t);

@@ -415,112 +415,117 @@ __global__ void psgrad_kernel(const FieldDev *__restrict__ fields, const int4 *_
     }
 }
 
-// dL/dh[u] = T0[u] + sum_i G_i[u]: one thread per polyphase index q = phi*N*N + m.
-__global__ void hgrad_kernel(const FieldDev *__restrict__ fields, const ChunkItem *__restrict__ chunks, int n_chunks,
-                             const float *__restrict__ gbuf, float *__restrict__ grad, const float *__restrict__ params) {
-    const int c = blockIdx.x;
+// dL/dh[u] = T0[u] + sum_i G_i[u] over the polyphase indexes q = phi*N*N + m.  A block takes a quarter
+// of a 256-pixel chunk: 64 pixels by kHgGroups groups of epochs (group g the epochs i = g mod 4 of
+// the whole quadruples, group 0 also the rest), whose sums are joined as (0 + 1) + (2 + 3).  A field
+// of few chunks is bound by the chain of each pixel's gathers over its epochs (rotated frames test 9
+// candidates per epoch): with one thread per pixel a 24-epoch field of 64 x 64 took 76 us on 64
+// blocks, with four 26 us on 256.
+constexpr int kHgGroups = 4, kHgPixels = 256 / kHgGroups;
+
+// the bilinear gather of one epoch's adjoint image at pixel (vx, vy)
+__device__ __forceinline__ float hgrad_rotated(const FieldDev &fd, const float *__restrict__ Gi, float2 cs, float2 sh,
+                                               int vx, int vy) {
+    // every u whose bilinear read (frame_point) has v in its cell; those u lie within 1.5 pixels of
+    // u0 + s + R (v - u0) on each axis
+    const int f = fd.f, N = fd.N, F = fd.F;
+    const float u0 = 0.5f * (float)(F - 1);
+    const float ex = (float)vx - u0, ey = (float)vy - u0;
+    const float cx = u0 + sh.x + (cs.x * ex - cs.y * ey), cy = u0 + sh.y + (cs.y * ex + cs.x * ey);
+    const int ux0 = max(0, (int)ceilf(cx - 1.5f)), ux1 = min(F - 1, (int)floorf(cx + 1.5f));
+    const int uy0 = max(0, (int)ceilf(cy - 1.5f)), uy1 = min(F - 1, (int)floorf(cy + 1.5f));
+    float gi = 0.f;
+    for (int uy = uy0; uy <= uy1; ++uy)
+        for (int ux = ux0; ux <= ux1; ++ux) {
+            const float2 qp = frame_point(F, cs, sh, ux, uy);
+            const float fx = floorf(qp.x), fy = floorf(qp.y);
+            const int a = vx - (int)fx, b = vy - (int)fy;
+            if ((unsigned)a > 1u || (unsigned)b > 1u) continue;
+            const float tx = qp.x - fx, ty = qp.y - fy;
+            const int uph = (uy % f) * f + ux % f;
+            gi += (b ? ty : 1.f - ty) * (a ? tx : 1.f - tx) *
+                  Gi[(long long)uph * N * N + (uy / f) * N + ux / f];
+        }
+    return gi;
+}
+
+__device__ __forceinline__ float hgrad_shifted(const FieldDev &fd, const float *__restrict__ Gi, const float *dl, int vx,
+                                               int vy) {
+    // T_i^T G_i: pixel v gathers G_i(v - n - (0 | 1)) with the read's weights
+    const int f = fd.f, N = fd.N, F = fd.F;
+    int nx, ny;
+    float tx, ty;
+    shift_split((float)f * dl[0], &nx, &tx);
+    shift_split((float)f * dl[1], &ny, &ty);
+    float gi = 0.f;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        const int uy = vy - ny - b;
+        if (uy < 0 || uy >= F) continue;
+        const float wy = b ? ty : 1.f - ty;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int ux = vx - nx - a;
+            if (ux < 0 || ux >= F) continue;
+            const int uph = (uy % f) * f + ux % f;
+            gi += wy * (a ? tx : 1.f - tx) * Gi[(long long)uph * N * N + (uy / f) * N + ux / f];
+        }
+    }
+    return gi;
+}
+
+__global__ void __launch_bounds__(256)
+hgrad_kernel(const FieldDev *__restrict__ fields, const ChunkItem *__restrict__ chunks, int n_chunks,
+             const float *__restrict__ gbuf, float *__restrict__ grad, const float *__restrict__ params) {
+    __shared__ float part[kHgGroups][kHgPixels];
+    const int c = blockIdx.x / kHgGroups, quarter = blockIdx.x % kHgGroups;
     if (c >= n_chunks) return;
     const ChunkItem ch = chunks[c];
     const FieldDev &fd = fields[ch.field];
     if (fd.mode != 0) return;  // fields in the frequency-domain form get dL/dh from fft_hgrad_kernel
-    const int q = ch.start + threadIdx.x;
-    const int f = fd.f, N = fd.N, F = fd.F;
-    if (q >= F * F) return;
+    const int px = threadIdx.x % kHgPixels, g = threadIdx.x / kHgPixels;
+    const int q = ch.start + quarter * kHgPixels + px;
+    const int f = fd.f, N = fd.N, F = fd.F, E = fd.E;
     const long long plane = (long long)f * f * N * N;
-    if (fd.rot) {
-        // dL/dh = sum_i W_i^T G_i: pixel v gathers every u whose bilinear read (frame_point) has v
-        // in its cell; those u lie within 1.5 pixels of u0 + s + R (v - u0) on each axis
-        const int ph = q / (N * N), m = q - ph * N * N;
-        const int vy = f * (m / N) + ph / f, vx = f * (m % N) + ph % f;
-        const float *cpar = params + fd.param_off + (long long)F * F + (long long)fd.E * fd.M + 2 * fd.M;
-        const float *Gb = gbuf + fd.gbuf_off;
-        const float u0 = 0.5f * (float)(F - 1);
-        float acc = 0.f;
-        for (int i = 0; i < fd.E; ++i) {
-            const float2 cs = fd.rot[i];
-            const float2 sh = fd.translate ? make_float2((float)f * cpar[2 * i], (float)f * cpar[2 * i + 1])
-                                           : make_float2(0.f, 0.f);
-            const float ex = (float)vx - u0, ey = (float)vy - u0;
-            const float cx = u0 + sh.x + (cs.x * ex - cs.y * ey), cy = u0 + sh.y + (cs.y * ex + cs.x * ey);
-            const int ux0 = max(0, (int)ceilf(cx - 1.5f)), ux1 = min(F - 1, (int)floorf(cx + 1.5f));
-            const int uy0 = max(0, (int)ceilf(cy - 1.5f)), uy1 = min(F - 1, (int)floorf(cy + 1.5f));
-            float gi = 0.f;
-            for (int uy = uy0; uy <= uy1; ++uy)
-                for (int ux = ux0; ux <= ux1; ++ux) {
-                    const float2 qp = frame_point(F, cs, sh, ux, uy);
-                    const float fx = floorf(qp.x), fy = floorf(qp.y);
-                    const int a = vx - (int)fx, b = vy - (int)fy;
-                    if ((unsigned)a > 1u || (unsigned)b > 1u) continue;
-                    const float tx = qp.x - fx, ty = qp.y - fy;
-                    const int uph = (uy % f) * f + ux % f;
-                    gi += (b ? ty : 1.f - ty) * (a ? tx : 1.f - tx) *
-                          Gb[(long long)i * plane + (long long)uph * N * N + (uy / f) * N + ux / f];
-                }
-            acc += gi;
-        }
-        const int u = vy * F + vx;
-        grad[fd.param_off + u] = acc + fd.starlet[(long long)fd.J * F * F + u];
-        return;
-    }
-    if (fd.translate) {
-        // dL/dh = sum_i T_i^T G_i: pixel v gathers G_i(v - n - (0 | 1)) with the read's weights
-        const int ph = q / (N * N), m = q - ph * N * N;
-        const int vy = f * (m / N) + ph / f, vx = f * (m % N) + ph % f;
-        const float *cpar = params + fd.param_off + (long long)F * F + (long long)fd.E * fd.M + 2 * fd.M;
-        const float *Gb = gbuf + fd.gbuf_off;
-        float acc = 0.f;
-        for (int i = 0; i < fd.E; ++i) {
-            int nx, ny;
-            float tx, ty;
-            shift_split((float)f * cpar[2 * i], &nx, &tx);
-            shift_split((float)f * cpar[2 * i + 1], &ny, &ty);
-            float gi = 0.f;
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const int uy = vy - ny - b;
-                if (uy < 0 || uy >= F) continue;
-                const float wy = b ? ty : 1.f - ty;
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    const int ux = vx - nx - a;
-                    if (ux < 0 || ux >= F) continue;
-                    const int uph = (uy % f) * f + ux % f;
-                    gi += wy * (a ? tx : 1.f - tx) *
-                          Gb[(long long)i * plane + (long long)uph * N * N + (uy / f) * N + ux / f];
-                }
-            }
-            acc += gi;
-        }
-        const int u = vy * F + vx;
-        grad[fd.param_off + u] = acc + fd.starlet[(long long)fd.J * F * F + u];
-        return;
-    }
-    const float *G = gbuf + fd.gbuf_off + q;
-    // four interleaved FP32 partial sums over the epochs, combined in a fixed order
-    // (the FP64 pipe of this GPU is far narrower than the FP32 one)
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    int i = 0;
-    for (; i + 4 <= fd.E; i += 4) {
-        s0 += G[(long long)i * plane];
-        s1 += G[(long long)(i + 1) * plane];
-        s2 += G[(long long)(i + 2) * plane];
-        s3 += G[(long long)(i + 3) * plane];
-    }
-    for (; i < fd.E; ++i) s0 += G[(long long)i * plane];
     const int ph = q / (N * N), m = q - ph * N * N;
-    const int my = m / N, mx = m - my * N;
-    const int u = (f * my + ph / f) * F + f * mx + ph % f;
-    const float *T0 = fd.starlet + (long long)fd.J * F * F;
-    grad[fd.param_off + u] = ((s0 + s1) + (s2 + s3)) + T0[u];
+    const int vy = f * (m / N) + ph / f, vx = f * (m % N) + ph % f;
+    const int quads = E / kHgGroups * kHgGroups;
+    float acc = 0.f;
+    if (q < F * F) {
+        const float *Gb = gbuf + fd.gbuf_off;
+        const float *dl = params + fd.param_off + (long long)F * F + (long long)E * fd.M + 2 * fd.M;
+        auto term = [&](int i) {
+            const float *Gi = Gb + (long long)i * plane;
+            if (fd.rot) {
+                const float2 sh = fd.translate ? make_float2((float)f * dl[2 * i], (float)f * dl[2 * i + 1])
+                                               : make_float2(0.f, 0.f);
+                return hgrad_rotated(fd, Gi, fd.rot[i], sh, vx, vy);
+            }
+            return fd.translate ? hgrad_shifted(fd, Gi, dl + 2 * i, vx, vy) : Gi[q];
+        };
+#pragma unroll 4
+        for (int i = g; i < quads; i += kHgGroups) acc += term(i);
+        if (g == 0)
+            for (int i = quads; i < E; ++i) acc += term(i);
+    }
+    part[g][px] = acc;
+    __syncthreads();
+    if (g != 0 || q >= F * F) return;
+    const int u = vy * F + vx;
+    grad[fd.param_off + u] =
+        ((part[0][px] + part[1][px]) + (part[2][px] + part[3][px])) + fd.starlet[(long long)fd.J * F * F + u];
 }
 
 // The moved channel's part of dL/d delta_i = f sum_u G_i(u) d(T h)(u)/d s, with d(T h)/d s_x =
 // -[(1 - t_y)(h(y0, x0 + 1) - h(y0, x0)) + t_y (h(y0 + 1, x0 + 1) - h(y0 + 1, x0))] (and the same with
 // the axes swapped), (x0, y0) = u + n.  Block (epoch, field); compensated FP32 sums in fixed order.
-__global__ void __launch_bounds__(256)
+// 1024 threads per block: with 256 a 24-epoch field's 24 blocks took 59 us, now 30 (64 pixels of gathers per
+// thread in a row).
+constexpr int kShiftThreads = 1024;
+__global__ void __launch_bounds__(kShiftThreads)
 hshift_grad_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params,
                    const float *__restrict__ gbuf, float *__restrict__ hs) {
-    __shared__ float4 s_red[8];
+    __shared__ float4 s_red[kShiftThreads / 32];
     const FieldDev &fd = fields[blockIdx.y];
     const int i = blockIdx.x;
     if (!fd.translate || fd.mode != 0 || i >= fd.E) return;
@@ -741,12 +746,12 @@ void launch_psgrad(const FieldDev *fields, const int4 *ps_items, int n, const fl
 
 void launch_hgrad(const FieldDev *fields, const ChunkItem *chunks, int n_chunks, const float *gbuf, float *grad,
                   const float *params, cudaStream_t st) {
-    hgrad_kernel<<<n_chunks, 256, 0, st>>>(fields, chunks, n_chunks, gbuf, grad, params);
+    hgrad_kernel<<<n_chunks * kHgGroups, 256, 0, st>>>(fields, chunks, n_chunks, gbuf, grad, params);
 }
 
 void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, const float *params, const float *gbuf,
                         float *hs, cudaStream_t st) {
-    hshift_grad_kernel<<<dim3(E_max, n_fields), 256, 0, st>>>(fields, params, gbuf, hs);
+    hshift_grad_kernel<<<dim3(E_max, n_fields), kShiftThreads, 0, st>>>(fields, params, gbuf, hs);
 }
 
 void launch_finalize(const FieldDev *fields, int n_fields, const double *chi_part, const double *se_part,
