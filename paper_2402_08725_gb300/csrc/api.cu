@@ -626,10 +626,9 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
             smem_fft = std::max(smem_fft, fft_pair_field_smem(L));
             // epoch pairs side by side: the widest group the kernel is compiled for at this size
             // (more than one pair only with at most one source) if its buffers fit, else one pair
-            int G = fd.M <= 1 && opt.gp_cap != 1 ? fft_pair_gpmax(L) : 1;
+            int G = opt.gp_cap != 1 ? fft_pair_gpmax(L, fd.M) : 1;
             if (G > 1 && fft_pair_smem_bytes(L, fd.M, fd.f, G) > g_fx_smem_limit) G = 1;
             fd.fft_G = G;
-            fd.fft_EB = fft_pair_zn(L);
             smem_fx = std::max(smem_fx, fft_pair_smem_bytes(L, fd.M, fd.f, G));
         } else if (pl->kind == SR_DECONV && !plain) {
             gbuf += (long long)fd.E * fd.f * fd.f * fd.N * fd.N;
@@ -1178,7 +1177,7 @@ sr_status sr_create_problem(const sr_problem_desc *desc, void *cuda_stream, sr_p
             if ((st = device_limits()) != SR_OK) return bail(st);
             int L = 0;
             const bool ok = d.n_sources <= kFftMaxSources && fft_size(d.data_n, p->Tk, p->tau_lo, &L) &&
-                            fft_pair_field_smem(L) <= g_fft_smem_limit && fft_pair_variant(L, d.n_sources, 1) &&
+                            fft_pair_field_smem(L) <= g_fft_smem_limit && fft_pair_variant(L, d.n_sources) &&
                             fft_pair_smem_bytes(L, d.n_sources, d.supersampling, 1) <= g_fx_smem_limit;
             // sizes beyond shared memory: the global-memory transforms of fft_big.cu
             const int tau_hi = p->tau_lo + p->Tk - 1;
@@ -1195,8 +1194,9 @@ sr_status sr_create_problem(const sr_problem_desc *desc, void *cuda_stream, sr_p
                 if ((st = A.alloc(&p->big_zt, E * npr * (size_t)p->Tk * L)) != SR_OK) return bail(st);
             } else if (ok) {
                 const size_t H = L / 2 + 1;
-                // rows padded to H + 1 (even), so that column pairs are 16-byte aligned
-                if ((st = A.alloc(&p->khat, E * d.supersampling * d.supersampling * (size_t)L * (H + 1))) != SR_OK)
+                // both epochs of a pair side by side, rows padded to H + 1
+                if ((st = A.alloc(&p->khat, 2 * ((E + 1) / 2) * d.supersampling * d.supersampling * (size_t)L *
+                                                (H + 1))) != SR_OK)
                     return bail(st);
             }
             if (ok || big) {
@@ -1970,7 +1970,7 @@ static sr_status batch_io_prepare(sr_batch *b) {
         os[i + 1] = os[i] + (long long)e.E * e.K * e.K;
         ok[i + 1] = ok[i] + (long long)e.E * e.f * e.f * e.Tk * e.Tk;
         if (p->khat && !p->fft_big)
-            for (int j = 0; j < e.E * ((e.f * e.f + 1) / 2); ++j) items.push_back(make_int2(i, j));
+            for (int j = 0; j < (e.E + 1) / 2 * e.f * e.f; ++j) items.push_back(make_int2(i, j));
     }
     // items grouped by transform size: one launch per size with that size's block
     std::stable_sort(items.begin(), items.end(), [&](const int2 &a, const int2 &c) {

@@ -52,14 +52,14 @@ struct FieldDev {
     int mode;
     int fft_L;
     const float2 *fft_tw;     // [L] exp(-2 pi i n / L)
-    // spectra in global memory are rows of L/2+2 (the last column a zero pad, so that column
-    // pairs are 16-byte aligned)
-    const float2 *fft_khat;   // [E][f*f][L][L/2+2] transforms of the folded kernels
+    // spectra in global memory are rows of L/2+2 (the last column a zero pad)
+    // transforms of the folded kernels: mode 1 [ceil(E/2)][f*f][L][L/2+2] of (re_a, re_b, im_a, im_b) of
+    // the epochs 2p and 2p + 1; mode 2 [E][f*f][L/2+1][L]
+    const float2 *fft_khat;
     long long fft_hhat_off;   // offset of the field's [f*f][L][L/2+2] h spectra in the plan buffer
     long long fft_acc_off;    // float2 offset of the field's chunk accumulators ([f*f][L][L/2+2] each)
     int fft_n_chunks;         // epoch chunks of the field
     int fft_G;                // epoch pairs transformed side by side by the chunk kernel (1, 2 or 4)
-    int fft_EB;               // float2 elements of one pair array of the transform kernels
     // point-source prior (Eq. 11, third term): 1 + index of the partner entry (a field's shadow
     // entry in the plan's point-source table, or a shadow entry's field), 0 for none
     int pts;

@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "cpack.cuh"
 #include "cplx.cuh"
 #include "ffsum.cuh"
 #include "kernels.cuh"
@@ -163,6 +164,106 @@ __device__ __forceinline__ void dft(float2 *v) {
     else if constexpr (R == 16) dft_pq<4, 4, INV>(v);
     else if constexpr (R == 24) dft_pq<8, 3, INV>(v);
     else if constexpr (R == 32) dft_pq<8, 4, INV>(v);
+    else static_assert(R == 2, "unsupported in-register DFT size");
+}
+
+// --- the same DFTs over packed value types (cpack.cuh) ------------------------------------------
+template <int R, bool INV, typename T>
+__device__ __forceinline__ T zroot(T v, int m) {  // v W_R^m (forward) or v W_R^-m, exact for quarter turns
+    if (m == 0) return v;
+    if ((4 * m) % R == 0) {
+        const int q = (4 * m) / R;  // W^m = (-i)^q
+        if (q == 2) {
+            zneg(v);
+            return v;
+        }
+        return (q == 1) != INV ? zmulni(v) : zmuli(v);
+    }
+    const float2 w = c_dtw[dtw_off(R) + m];
+    return INV ? zmulwc(v, w) : zmulw(v, w);
+}
+
+template <int R, bool INV, typename T>
+__device__ __forceinline__ void zdft(T *v);
+
+template <int P, int Q, bool INV, typename T>
+__device__ __forceinline__ void zdft_pq(T *v) {  // as dft_pq
+    constexpr int R = P * Q;
+    T a[R];
+#pragma unroll
+    for (int n2 = 0; n2 < Q; ++n2) {
+        T t[P];
+#pragma unroll
+        for (int n1 = 0; n1 < P; ++n1) t[n1] = v[Q * n1 + n2];
+        zdft<P, INV>(t);
+#pragma unroll
+        for (int k1 = 0; k1 < P; ++k1) a[k1 * Q + n2] = zroot<R, INV>(t[k1], n2 * k1);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < P; ++k1) {
+        T t[Q];
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) t[n2] = a[k1 * Q + n2];
+        zdft<Q, INV>(t);
+#pragma unroll
+        for (int k2 = 0; k2 < Q; ++k2) v[k1 + P * k2] = t[k2];
+    }
+}
+
+template <int R, bool INV, typename T>
+__device__ __forceinline__ void zdft(T *v) {
+    if constexpr (R == 1) {
+    } else if constexpr (R == 2) {
+        const T a = v[0], b = v[1];
+        v[0] = zadd(a, b);
+        v[1] = zsub(a, b);
+    } else if constexpr (R == 3) {
+        constexpr float s = INV ? 0.866025403784438647f : -0.866025403784438647f;  // sin(-+2 pi / 3)
+        const T a = v[0], t = zadd(v[1], v[2]), u = zsub(v[1], v[2]);
+        v[0] = zadd(a, t);
+        const T m = zaxpy(-0.5f, t, a);
+        v[1] = zaxpyi(s, u, m);
+        v[2] = zaxpyi(-s, u, m);
+    } else if constexpr (R == 4) {
+        const T a = zadd(v[0], v[2]), b = zsub(v[0], v[2]), c = zadd(v[1], v[3]), d = zsub(v[1], v[3]);
+        v[0] = zadd(a, c);
+        v[2] = zsub(a, c);
+        v[1] = INV ? zaddi(b, d) : zsubi(b, d);
+        v[3] = INV ? zsubi(b, d) : zaddi(b, d);
+    } else if constexpr (R == 5) {
+        constexpr float c1 = 0.309016994374947424f, c2 = -0.809016994374947424f;  // cos 2pi/5, cos 4pi/5
+        constexpr float s1 = INV ? 0.951056516295153572f : -0.951056516295153572f;  // sin(-+2pi/5)
+        constexpr float s2 = INV ? 0.587785252292473129f : -0.587785252292473129f;  // sin(-+4pi/5)
+        const T a = v[0], t1 = zadd(v[1], v[4]), u1 = zsub(v[1], v[4]), t2 = zadd(v[2], v[3]), u2 = zsub(v[2], v[3]);
+        v[0] = zadd(zadd(a, t1), t2);
+        const T m1 = zaxpy(c2, t2, zaxpy(c1, t1, a)), m2 = zaxpy(c1, t2, zaxpy(c2, t1, a));
+        const T q1 = zaxpy(s2, u2, zscale(s1, u1)), q2 = zaxpy(-s1, u2, zscale(s2, u1));
+        v[1] = zaddi(m1, q1);
+        v[4] = zsubi(m1, q1);
+        v[2] = zaddi(m2, q2);
+        v[3] = zsubi(m2, q2);
+    } else if constexpr (R == 7) {
+        constexpr float c1 = 0.623489801858733530f, c2 = -0.222520933956314404f, c3 = -0.900968867902419126f;
+        constexpr float s1 = 0.781831482468029809f, s2 = 0.974927912181823607f, s3 = 0.433883739117558120f;
+        const T a = v[0];
+        const T t1 = zadd(v[1], v[6]), u1 = zsub(v[1], v[6]), t2 = zadd(v[2], v[5]), u2 = zsub(v[2], v[5]);
+        const T t3 = zadd(v[3], v[4]), u3 = zsub(v[3], v[4]);
+        v[0] = zadd(zadd(a, t1), zadd(t2, t3));
+        const float C[3][3] = {{c1, c2, c3}, {c2, c3, c1}, {c3, c1, c2}};     // cos(2 pi m j / 7)
+        const float S[3][3] = {{s1, s2, s3}, {s2, -s3, -s1}, {s3, -s1, s2}};  // sin(2 pi m j / 7)
+#pragma unroll
+        for (int m = 1; m <= 3; ++m) {
+            const float *cm = C[m - 1], *sm = S[m - 1];
+            const T re = zaxpy(cm[2], t3, zaxpy(cm[1], t2, zaxpy(cm[0], t1, a)));
+            const T q = zaxpy(sm[2], u3, zaxpy(sm[1], u2, zscale(sm[0], u1)));
+            v[m] = INV ? zaddi(re, q) : zsubi(re, q);
+            v[7 - m] = INV ? zsubi(re, q) : zaddi(re, q);
+        }
+    } else if constexpr (R == 6) zdft_pq<2, 3, INV>(v);
+    else if constexpr (R == 8) zdft_pq<2, 4, INV>(v);
+    else if constexpr (R == 9) zdft_pq<3, 3, INV>(v);
+    else if constexpr (R == 10) zdft_pq<2, 5, INV>(v);
+    else if constexpr (R == 16) zdft_pq<4, 4, INV>(v);
     else static_assert(R == 2, "unsupported in-register DFT size");
 }
 
@@ -377,15 +478,22 @@ __device__ __forceinline__ unsigned long long l2_policy_first() {
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
-// read-only loads (data not written during the kernel)
+// Read-only loads (data not written during the kernel), read once or twice by one SM: not kept in the
+// L1.  Volatile, so that a batch of them is issued where it is written, ahead of its use.
 __device__ __forceinline__ float2 ldg_hint(const float2 *p, unsigned long long pol) {
     float2 v;
-    asm("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(pol));
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float4 ldg_hint(const float4 *p, unsigned long long pol) {
+    float4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(pol));
     return v;
 }
 __device__ __forceinline__ float ldg_hint(const float *p, unsigned long long pol) {
     float v;
-    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
     return v;
 }
 // The accumulator: volatile, so that its loads and stores keep their program order among

@@ -55,6 +55,36 @@ __device__ void split_store(const float2 *Z, float2 *out_a, float2 *out_b, int s
     }
 }
 
+// The same for the two epochs of a kernel-spectra pair, side by side: out[ky][kx] = (re_a, re_b, im_a,
+// im_b); b zero without a second epoch.
+template <int L>
+__device__ void split_store_pair(const float2 *Z, float4 *out, bool hasb, int sh, const float2 *tw) {
+    using G = Pr<L>;
+    constexpr int H = G::H, HP = G::HP, P = G::P;
+    const int rows = blockDim.x / HP;  // rows in parallel
+    const int kx = threadIdx.x % HP, ty = threadIdx.x / HP;
+    if (ty >= rows) return;
+    const bool live = kx < H;
+    const int cx = live ? kcol<L>(kx) : 0, cxm = live ? kcol<L>(neg_mod(kx, L)) : 0;
+    const int wx = (int)(((long long)kx * sh) % L);
+    const int wstep = (int)(((long long)rows * sh) % L);
+    int wi = (int)(((long long)ty * sh) % L) + wx;
+    if (wi >= L) wi -= L;
+    for (int ky = ty; ky < L; ky += rows) {
+        float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
+        if (live) {
+            const float2 A = Z[krow<L>(ky) * P + cx];
+            const float2 B = Z[krow<L>(neg_mod(ky, L)) * P + cxm];
+            const float2 w = tw[wi];
+            xa = cmul(make_float2(0.5f * (A.x + B.x), 0.5f * (A.y - B.y)), w);
+            if (hasb) xb = cmul(make_float2(0.5f * (A.y + B.y), 0.5f * (B.x - A.x)), w);
+        }
+        out[ky * HP + kx] = make_float4(xa.x, xb.x, xa.y, xb.y);
+        wi += wstep;
+        if (wi >= L) wi -= L;
+    }
+}
+
 // The forward transform along y of a pair whose rows y >= ylim are zero, with ylim <= L/2
 // (NZ = 8) or <= L/4 (NZ = 4) and R1 = 16: pass A's 16-point DFTs see non-zero inputs only at
 // n1 < NZ, so their first radix-4 stage reduces to one (NZ = 4) or two (NZ = 8) terms; pass B is
@@ -117,10 +147,11 @@ __device__ __noinline__ void cols_fwd_lead(float2 *Z, int ylim, const float2 *TW
     __syncthreads();
 }
 
-// Spectra of the folded PSF kernels (at set_psfs): item = epoch * n_pairs + pair of phases.  The
-// phase kernel kappa_phi (Tk x Tk, taps tau_lo .. tau_lo + Tk - 1 on each axis, Tk <= L) belongs on
-// the L x L circle with tap tau at tau mod L.  It is placed instead at tau - tau_lo, so that the
-// row passes touch only its Tk rows, and the shift is restored on the spectrum (shift theorem):
+// Spectra of the folded PSF kernels (at set_psfs): item = epoch pair * f^2 + phase, the two epochs'
+// kernels of the phase as one complex image.  The phase kernel kappa_phi (Tk x Tk, taps tau_lo ..
+// tau_lo + Tk - 1 on each axis, Tk <= L) belongs on the L x L circle with tap tau at tau mod L.  It is
+// placed instead at tau - tau_lo, so that the row passes touch only its Tk rows, and the shift is
+// restored on the spectrum (shift theorem):
 //   Khat[ky][kx] = W_L^((ky + kx) tau_lo) Khat'[ky][kx],   W_L = exp(-2 pi i / L).
 template <int L>
 __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__restrict__ kappa,
@@ -129,12 +160,11 @@ __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__
     constexpr int P = G::P, HP = G::HP;
     float2 *Z = pr_dyn, *TWL = Z + G::ZN;
     load_twl<L>(TWL, fd.fft_tw);
-    const int nph = fd.f * fd.f, npr = (nph + 1) / 2;
-    const int i = item / npr, q = item - i * npr;
-    const int pa = 2 * q, pb = 2 * q + 1;
+    const int nph = fd.f * fd.f;
+    const int pr = item / nph, ph = item - pr * nph;
     const int Tk = fd.Tk;
-    const float *ka = kappa + ((long long)i * nph + pa) * Tk * Tk;
-    const float *kb = pb < nph ? ka + Tk * Tk : nullptr;
+    const float *ka = kappa + ((long long)(2 * pr) * nph + ph) * Tk * Tk;
+    const float *kb = 2 * pr + 1 < fd.E ? ka + (long long)nph * Tk * Tk : nullptr;
     for (int t = threadIdx.x; t < Tk * Tk; t += blockDim.x) {
         const int y = t / Tk, x = t - y * Tk;
         Z[y * P + pcol<L>(x)] = make_float2(ka[t], kb ? kb[t] : 0.f);
@@ -149,14 +179,14 @@ __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__
         cols_fwd<L>(Z, 1, Tk, TWL);
     }
     const int sh = ((fd.tau_lo % L) + L) % L;  // tau_lo mod L
-    float2 *out = khat + ((long long)i * nph + pa) * L * HP;
-    split_store<L>(Z, out, kb ? out + L * HP : nullptr, sh, fd.fft_tw);
+    float4 *out = reinterpret_cast<float4 *>(khat) + (long long)item * L * HP;
+    split_store_pair<L>(Z, out, kb != nullptr, sh, fd.fft_tw);
     __syncthreads();
 }
 
 __global__ void __launch_bounds__(kFftThreads, 1)
 fft_kappa_pair_kernel(FieldDev fd, const float *__restrict__ kappa, float2 *__restrict__ khat) {
-    const int n_items = fd.E * ((fd.f * fd.f + 1) / 2);
+    const int n_items = (fd.E + 1) / 2 * fd.f * fd.f;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         switch (fd.fft_L) {
 #define SR_PR_KCASE(LL)                                 \
@@ -171,8 +201,8 @@ fft_kappa_pair_kernel(FieldDev fd, const float *__restrict__ kappa, float2 *__re
     }
 }
 
-// The kernel spectra of many problems in one launch: items[j] = (table entry, epoch * n_pairs +
-// pair); every block takes items in turn (the spectra live at each entry's fft_khat).
+// The kernel spectra of many problems in one launch: items[j] = (table entry, epoch pair * f^2 +
+// phase); every block takes items in turn (the spectra live at each entry's fft_khat).
 __global__ void __launch_bounds__(kFftThreads, 1)
 fft_kappa_pair_batch_kernel(const FieldDev *__restrict__ fields, const int2 *__restrict__ items, int n_items) {
     for (int j = blockIdx.x; j < n_items; j += gridDim.x) {
@@ -457,7 +487,7 @@ sr_status launch_fft_kappa_pair_batch(const FieldDev *fields, const int2 *items,
 }
 
 void launch_fft_kappa_pair(const FieldDev &fd, const float *kappa, float2 *khat, cudaStream_t st) {
-    const int n_items = fd.E * ((fd.f * fd.f + 1) / 2);
+    const int n_items = (fd.E + 1) / 2 * fd.f * fd.f;
     const int smem = fft_pair_field_smem(fd.fft_L);
     int threads = 0, occ = 0;
     kappa_block(fft_kappa_pair_kernel, smem, &threads, &occ);

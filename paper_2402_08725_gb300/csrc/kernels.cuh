@@ -42,13 +42,14 @@ int fft_pair_next(int need);  // smallest listed size >= need, 0 if none
 int fft_pair_zn(int L);       // float2 elements of one pair array
 int fft_pair_smem_bytes(int L, int M, int f, int GP);  // chunk kernel, GP epoch pairs per group
 int fft_pair_field_smem(int L);                        // per-field and per-PSF kernels
-bool fft_pair_variant(int L, int M, int GP);           // the chunk kernel is compiled for it
-int fft_pair_gpmax(int L);                             // widest group of pairs (one source)
+bool fft_pair_variant(int L, int M);                   // the chunk kernel takes M sources at this size
+int fft_pair_gpmax(int L, int M);                      // epoch pairs per group
 sr_status configure_fft_pair(int optin, int *chunk_limit, int *field_limit);
 sr_status configure_fft_pair_field(int optin, int *field_limit);  // called by configure_fft_pair
-// spectra of a problem's folded kernels (set_psfs): [E][f*f][L][L/2+2], the pad column zero
+// spectra of a problem's folded kernels (set_psfs): [ceil(E/2)][f*f][L][L/2+2] of (re_a, re_b, im_a,
+// im_b) for epochs 2p and 2p + 1 (zero for a missing last one), the pad column zero
 void launch_fft_kappa_pair(const FieldDev &fd, const float *kappa, float2 *khat, cudaStream_t st);
-// the same for (entry, epoch * pairs + pair of phases) items of a table whose entries all have
+// the same for (entry, epoch pair * f^2 + phase) items of a table whose entries all have
 // transform size L (each entry's kappa and fft_khat), a persistent grid over n_sms SMs
 sr_status launch_fft_kappa_pair_batch(const FieldDev *fields, const int2 *items, int n_items, int L, int n_sms,
                                       cudaStream_t st);
