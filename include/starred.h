@@ -354,9 +354,9 @@ int sr_batch_field_form(const sr_batch *b, int i);
  * computed).  The per-epoch kernel takes work items of epochs_per_item
  * consecutive epochs of one field (each with its own accumulator of adjoint
  * spectra) and transforms pairs_per_group = 1 epoch pair at a time, or (0) the
- * widest group of pairs compiled for the field's transform size.  By default a
- * batch takes as many epochs per item as keep at least two items per SM (even,
- * 2 .. 16).  sr_batch_set_schedule rebuilds the batch's plan with the given
+ * widest group of pairs of the field's transform size.  By default the epochs
+ * per item (even, 2 .. 16) are those whose items, by a cost model, finish
+ * first on the GPU's SMs.  sr_batch_set_schedule rebuilds the batch's plan with the given
  * schedule (epochs_per_item 0 or even in 2 .. 16; pairs_per_group 0 or 1;
  * SR_ERR_ARG otherwise); it synchronises the batch's stream and drops its
  * captured optimiser graph.  Results differ between schedules only by the

@@ -7,10 +7,12 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -165,6 +167,43 @@ using namespace sr;
 // ------------------------------------------------------------------------------------------
 // Execution plan: fields, work lists and scratch for one evaluation of one or many fields.
 // ------------------------------------------------------------------------------------------
+// Work of an evaluation that needs only part of what the evaluation's stream does runs on a stream of
+// its own between a fork and a join: the priors read only the parameters and write their own
+// buffers; the sources' gradients read the adjoint images while dL/dh is formed from them.  The owner's
+// stream orders a plan's evaluations, and both events tie the branch to it.  Not open (no stream): the
+// work stays in order on the evaluation's stream.
+struct Branch {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t forked = nullptr, joined = nullptr;
+    ~Branch() {
+        if (forked) cudaEventDestroy(forked);
+        if (joined) cudaEventDestroy(joined);
+        if (stream) cudaStreamDestroy(stream);
+    }
+    sr_status open() {
+        SR_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
+        SR_CUDA(cudaEventCreateWithFlags(&forked, cudaEventDisableTiming));
+        SR_CUDA(cudaEventCreateWithFlags(&joined, cudaEventDisableTiming));
+        return SR_OK;
+    }
+    // the branch's stream, ordered after everything queued on `st` so far; `st` itself when not open
+    // (or when the fork fails: the order is then kept)
+    cudaStream_t fork(cudaStream_t st) {
+        if (!stream) return st;
+        if (cudaEventRecord(forked, st) != cudaSuccess || cudaStreamWaitEvent(stream, forked, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return st;
+        }
+        return stream;
+    }
+    // orders `st` after the branch (a failure is left for the evaluation's error check)
+    void join(cudaStream_t branch, cudaStream_t st) {
+        if (branch == st) return;
+        cudaEventRecord(joined, branch);
+        cudaStreamWaitEvent(st, joined, 0);
+    }
+};
+
 struct Plan {
     int kind = SR_DECONV;
     bool plain = false;
@@ -227,41 +266,15 @@ struct Plan {
     bool profiling = false;
     int prof_count = 0;
     std::vector<cudaEvent_t> prof_ev;
-    // The prior branch: the starlet levels (and the point-source prior) read only the parameters
-    // and write their own buffers, so they run on this stream beside the chi^2 branch, between a
-    // fork at the start of the evaluation and a join before dL/dh (NULL: everything in order on
-    // the evaluation's stream).  A plan's evaluations are ordered by its owner's stream, which
-    // both events tie the branch to, so one stream per plan is enough.
-    cudaStream_t side = nullptr;
-    cudaEvent_t side_fork = nullptr, side_join = nullptr;
+    // Branches of the evaluation beside its own stream (see Branch): the starlet prior on h, the
+    // point-source prior, and the sources' gradients
+    Branch prior, pts, src;
     DevArena arena;
     ~Plan() {
         if (graph) cudaGraphExecDestroy(graph);
         for (cudaEvent_t e : prof_ev) cudaEventDestroy(e);
-        if (side_fork) cudaEventDestroy(side_fork);
-        if (side_join) cudaEventDestroy(side_join);
-        if (side) cudaStreamDestroy(side);
     }
 };
-
-// The stream of the evaluation's prior branch, ordered after everything queued on `st` so far;
-// `st` itself when the plan has no branch (or the fork fails: the order is then kept).
-static cudaStream_t fork_prior(Plan *pl, cudaStream_t st) {
-    if (!pl->side) return st;
-    if (cudaEventRecord(pl->side_fork, st) != cudaSuccess ||
-        cudaStreamWaitEvent(pl->side, pl->side_fork, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return st;
-    }
-    return pl->side;
-}
-
-// Orders `st` after the branch.
-static void join_prior(Plan *pl, cudaStream_t branch, cudaStream_t st) {
-    if (branch == st) return;
-    cudaEventRecord(pl->side_join, branch);
-    cudaStreamWaitEvent(st, pl->side_join, 0);
-}
 
 struct sr_problem {
     sr_problem_desc desc{};
@@ -519,6 +532,67 @@ struct PlanOptions {
 
 static bool field_uses_fft(sr_problem *p, const PlanOptions &opt);
 
+// Default epochs per work item of the transform form (even, 2 .. kFftChunk): the shortest time to
+// finish the items on one block per SM, longest first, plus the traffic of their accumulators.
+// An item costs its epoch pairs' transforms (measured: 8 to 11 cycles per point of the L x L pair at
+// f = 2, by the phases above that, and 0.45 more per further source; 0.6 of it once per group of pairs,
+// whose passes it shares) and a fixed part; an accumulator is written, read back and added at about
+// 400 bytes a clock over the GPU.  Against "as many epochs as keep
+// two items per SM" (us per evaluation): 1000 epochs of 32 x 32 157 -> 102 (8 epochs instead of 2: 125
+// items finish together, 500 leave a fourth of a round and 4 times the accumulators), 500 of 48 x 48
+// 123 -> 94, 24 fields of 10-60 epochs 269 -> 193; 300 of 64 x 64 keeps 2.  Fields that fill the GPU several
+// times at the longest items take those.
+static int default_chunk(sr_problem *const *probs, int n, int epoch_limit) {
+    struct Shape {
+        double pair, acc;  // cycles of a pair; accumulator bytes
+        int epochs, group;
+    };
+    std::vector<Shape> sh;
+    const int sms = std::max(g_num_sms, 1);
+    long long longest = 0;
+    for (int i = 0; i < n; ++i) {
+        const sr_problem *p = probs[i];
+        if (!p->fft_ok || p->fft_big) continue;
+        const double L = p->fft_L, nph = (double)p->desc.supersampling * p->desc.supersampling;
+        const int E = epoch_limit > 0 ? std::min(p->desc.n_epochs, epoch_limit) : p->desc.n_epochs;
+        sh.push_back({9.0 * L * L * (0.25 + 0.1875 * nph) * (1.0 + 0.45 * std::max(0, p->desc.n_sources - 1)),
+                      nph * L * (L / 2 + 2) * 8.0, E, fft_pair_gpmax(p->fft_L, p->desc.n_sources)});
+        longest += (E + kFftChunk - 1) / kFftChunk;
+    }
+    if (longest >= 4LL * sms) return kFftChunk;
+    std::stable_sort(sh.begin(), sh.end(), [](const Shape &a, const Shape &b) { return a.pair > b.pair; });
+    int best = 2;
+    double best_t = 0.0;
+    for (int c = 2; c <= kFftChunk; c += 2) {
+        std::vector<double> items;
+        double bytes = 0.0;
+        for (const Shape &s : sh)
+            for (int e = 0; e < s.epochs; e += c) {
+                const int pairs = (std::min(c, s.epochs - e) + 1) / 2, groups = (pairs + s.group - 1) / s.group;
+                items.push_back((0.6 * groups + 0.4 * pairs) * s.pair + 4000.0);
+                bytes += 2.0 * s.acc;
+            }
+        std::sort(items.begin(), items.end(), [](double a, double b) { return a > b; });
+        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+        double end = 0.0;
+        for (double t : items) {
+            double at = 0.0;
+            if ((int)free_at.size() >= sms) {
+                at = free_at.top();
+                free_at.pop();
+            }
+            free_at.push(at + t);
+            end = std::max(end, at + t);
+        }
+        const double total = end + bytes / 400.0;
+        if (c == 2 || total < std::min(0.95 * best_t, best_t - 20000.0)) {  // 10 us at least
+            best = c;
+            best_t = total;
+        }
+    }
+    return best;
+}
+
 // Build the evaluation plan of `n` problems of the same kind.
 static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plain,
                             const PlanOptions &opt = PlanOptions()) {
@@ -544,16 +618,7 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
     std::vector<ChunkItem> sh_chunks;
     long long pbar_len = 0, l1pts = 0, ptsslot = 0;
     long long hs_len = 0;
-    // epochs per work item of the transform form: by default as many as keep at least two items per
-    // SM (even, 2 .. kFftChunk), so that a single long field spreads over the GPU
-    int chunk = opt.chunk;
-    if (chunk <= 0) {
-        long long ep = 0;
-        for (int i = 0; i < n; ++i)
-            if (probs[i]->fft_ok && !probs[i]->fft_big)
-                ep += opt.epoch_limit > 0 ? std::min(probs[i]->desc.n_epochs, opt.epoch_limit) : probs[i]->desc.n_epochs;
-        chunk = (int)std::min<long long>(kFftChunk, std::max<long long>(2, ep / (2LL * std::max(g_num_sms, 1)))) & ~1;
-    }
+    int chunk = opt.chunk > 0 ? opt.chunk : default_chunk(probs, n, opt.epoch_limit);
     chunk = std::max(2, std::min(kFftChunk, chunk)) & ~1;
     pl->chunk = chunk;
     pl->gp_cap = opt.gp_cap;
@@ -853,9 +918,9 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
         }
     }
     if (!plain && opt.grid_limit == 0) {  // (the form autotuner times its plans in order)
-        SR_CUDA(cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking));
-        SR_CUDA(cudaEventCreateWithFlags(&pl->side_fork, cudaEventDisableTiming));
-        SR_CUDA(cudaEventCreateWithFlags(&pl->side_join, cudaEventDisableTiming));
+        if ((st = pl->prior.open()) != SR_OK) return st;
+        if (pl->n_sh > 0 && (st = pl->pts.open()) != SR_OK) return st;
+        if (pl->n_ps > 0 && (st = pl->src.open()) != SR_OK) return st;
     }
     return SR_OK;
 }
@@ -866,11 +931,11 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
     int n = 0;
     if (pl->kind == SR_PSF) {
         const FieldDev &hf = pl->h_fields[0];
-        cudaStream_t prior = fork_prior(pl, st);
-        n += launch_psf_chi(pl->d_fields, hf, params, pl->psf, st);
+        cudaStream_t prior = pl->prior.fork(st);
         n += launch_starlet(pl->d_fields, 1, hf.F, starlet_forms_single(hf.F, hf.J, hf.Wmap != nullptr), pl->d_chunks,
                             pl->n_chunks, hf.J, params, pl->l1_part, prior);
-        join_prior(pl, prior, st);
+        n += launch_psf_chi(pl->d_fields, hf, params, pl->psf, st);
+        pl->prior.join(prior, st);
         n += launch_psf_finish(pl->d_fields, hf, params, grad, pl->psf, pl->l1_part, pl->losses, pl->total, st);
         return n;
     }
@@ -880,7 +945,20 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
                                pl->l1_part, pl->losses, pl->total, st);
         return n;
     }
-    cudaStream_t prior = fork_prior(pl, st);  // launched after the chi^2 branch, whose chain is the longer one
+    // The priors run beside the h spectra when they are one launch each (clusters), before the chunk
+    // kernel takes every SM (300 epochs of 64 x 64: 153 us an evaluation when launched after it);
+    // level by level they are launched after the chi^2 kernels, whose chain is the longer one.
+    cudaStream_t prior = pl->prior.fork(st), pts = pl->n_sh > 0 ? pl->pts.fork(st) : st;
+    auto launch_priors = [&]() {
+        n += launch_starlet(pl->d_fields, pl->n_fields, pl->Fmax, pl->starlet_forms, pl->d_chunks, pl->n_chunks,
+                            pl->Jmax, params, pl->l1_part, prior);
+        if (pl->n_sh > 0)
+            n += launch_pts_prior(pl->d_sh, pl->d_fields, pl->n_sh, pl->sh_Fmax, pl->sh_Mmax, pl->sh_starlet_forms,
+                                  pl->d_sh_chunks, pl->n_sh_chunks, pl->sh_Jmax, params, pl->abar, pl->pbar, pl->l1_pts,
+                                  pl->pts_g, pts);
+    };
+    const bool early = (pl->starlet_forms & kStarletClusterBit) != 0;
+    if (early) launch_priors();
     cudaMemsetAsync(pl->d_counters, 0, 4 * sizeof(int), st);
     cudaEvent_t *ev = nullptr;
     if (pl->profiling && !pl->prof_ev.empty()) {
@@ -909,27 +987,28 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
         n += 2;
     }
     for (size_t b = 0; b < pl->big_fields.size(); ++b)
-        n += launch_big_eval(pl->h_fields[pl->big_fields[b]], params, pl->big_buf[b], pl->ebuf, pl->gbuf, pl->chi_part,
-                             pl->se_part, st);
-    if (ev) cudaEventRecord(ev[3], st);
+        n += launch_big_model(pl->h_fields[pl->big_fields[b]], params, pl->big_buf[b], pl->ebuf, pl->chi_part,
+                              pl->se_part, st);
+    cudaStream_t src = st;
     if (pl->n_ps > 0) {
-        launch_psgrad(pl->d_fields, pl->d_ps, pl->n_ps, params, pl->gbuf, pl->ps_da, pl->ps_du, st);
+        src = pl->src.fork(st);
+        for (size_t b = 0; b < pl->big_fields.size(); ++b)
+            n += launch_big_window(pl->h_fields[pl->big_fields[b]], params, pl->ebuf, pl->gbuf, src);
+        launch_psgrad(pl->d_fields, pl->d_ps, pl->n_ps, params, pl->gbuf, pl->ps_da, pl->ps_du, src);
         ++n;
     }
-    n += launch_starlet(pl->d_fields, pl->n_fields, pl->Fmax, pl->starlet_forms, pl->d_chunks, pl->n_chunks, pl->Jmax,
-                        params, pl->l1_part, prior);
-    if (pl->n_sh > 0)
-        n += launch_pts_prior(pl->d_sh, pl->d_fields, pl->n_sh, pl->sh_Fmax, pl->sh_Mmax, pl->sh_starlet_forms,
-                              pl->d_sh_chunks, pl->n_sh_chunks, pl->sh_Jmax, params, pl->abar, pl->pbar, pl->l1_pts,
-                              pl->pts_g, prior);
-    join_prior(pl, prior, st);
+    if (pl->hs) {
+        launch_hshift_grad(pl->d_fields, pl->n_fields, pl->hs_Emax, params, pl->gbuf, pl->hs, src);
+        ++n;
+    }
+    for (size_t b = 0; b < pl->big_fields.size(); ++b)
+        n += launch_big_adj(pl->h_fields[pl->big_fields[b]], pl->big_buf[b], st);
+    if (ev) cudaEventRecord(ev[3], st);
+    if (!early) launch_priors();
+    pl->prior.join(prior, st);
     if (pl->n_items > 0) {
         launch_hgrad(pl->d_fields, pl->d_chunks, pl->n_chunks, pl->gbuf, grad, params, st);
         ++n;
-        if (pl->hs) {
-            launch_hshift_grad(pl->d_fields, pl->n_fields, pl->hs_Emax, params, pl->gbuf, pl->hs, st);
-            ++n;
-        }
     }
     if (pl->n_fft_items > 0) {
         n += launch_fft_hgrad_pair(pl->d_fields, pl->d_fft_fields, pl->n_fft_fields, pl->max_pairs, pl->smem_fft,
@@ -937,9 +1016,10 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
     }
     for (size_t b = 0; b < pl->big_fields.size(); ++b)
         n += launch_big_hgrad(pl->h_fields[pl->big_fields[b]], pl->big_buf[b], grad, st);
-    launch_finalize(pl->d_fields, pl->n_fields, pl->chi_part, pl->se_part, pl->l1_part, pl->ps_da, pl->ps_du, grad,
+    pl->pts.join(pts, st);
+    pl->src.join(src, st);
+    n += launch_finalize(pl->d_fields, pl->n_fields, pl->chi_part, pl->se_part, pl->l1_part, pl->ps_da, pl->ps_du, grad,
                     pl->losses, pl->total, st, pl->n_sh > 0 ? pl->d_sh : nullptr, pl->l1_pts, pl->pts_g, pl->hs);
-    n += 2;
     return n;
 }
 

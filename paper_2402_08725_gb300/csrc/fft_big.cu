@@ -685,8 +685,8 @@ static int big_spectra_t(const FieldDev &fd, const float *params, int mode, floa
 }
 
 template <int L>
-static int big_eval_t(const FieldDev &fd, const float *params, const BigBuffers &bb, float *ebuf, float *gbuf,
-                      double *chi_part, double *se_part, cudaStream_t st) {
+static int big_model_t(const FieldDev &fd, const float *params, const BigBuffers &bb, float *ebuf, double *chi_part,
+                       double *se_part, cudaStream_t st) {
     int n = big_spectra_t<L>(fd, params, 0, bb.zb, bb.zt, bb.fhat, st);
     const int H = L / 2 + 1, N = fd.N, np = (fd.E + 1) / 2;
     const dim3 cgrid((H + kBgItems - 1) / kBgItems, np), rgrid((N + kBgRows - 1) / kBgRows, np);
@@ -698,21 +698,20 @@ static int big_eval_t(const FieldDev &fd, const float *params, const BigBuffers 
     transpose(bb.zt, bb.zb, L, N, np, st);
     big_rows_kernel<L, BG_RESID_ROWS><<<rgrid, kBgThreads, bg_smem<L>(), st>>>(fd, bb.zb, params, ebuf, chi_part,
                                                                               se_part, nullptr);
+    return n + 3;
+}
+
+template <int L>
+static int big_adj_t(const FieldDev &fd, const BigBuffers &bb, cudaStream_t st) {
+    const int H = L / 2 + 1, N = fd.N, np = (fd.E + 1) / 2;
     transpose(bb.zb, bb.zt, N, L, np, st);
     BgArgs b{};
     b.zt_in = bb.zt;
     b.khat = fd.fft_khat;
     b.acc = bb.acc;
     b.ny = N;
-    big_cols_kernel<L, BG_ADJ><<<cgrid, kBgThreads, bg_smem<L>(), st>>>(fd, b);
-    n += 5;
-    if (fd.M > 0) {
-        const int nph = fd.f * fd.f;
-        big_window_adj_kernel<<<fd.E * fd.M * nph, kWinThreads, fft_big_window_smem(fd.Tk, fd.f), st>>>(fd, params, ebuf,
-                                                                                                      gbuf);
-        ++n;
-    }
-    return n;
+    big_cols_kernel<L, BG_ADJ><<<dim3((H + kBgItems - 1) / kBgItems, np), kBgThreads, bg_smem<L>(), st>>>(fd, b);
+    return 2;
 }
 
 template <int L>
@@ -741,14 +740,33 @@ int launch_big_kappa(const FieldDev &fd, float2 *zb, float2 *zt, cudaStream_t st
     }
 }
 
-int launch_big_eval(const FieldDev &fd, const float *params, const BigBuffers &bb, float *ebuf, float *gbuf,
-                    double *chi_part, double *se_part, cudaStream_t st) {
+int launch_big_model(const FieldDev &fd, const float *params, const BigBuffers &bb, float *ebuf, double *chi_part,
+                     double *se_part, cudaStream_t st) {
     switch (fd.fft_L) {
 #define SR_BG_E(LL) \
     case LL:        \
-        return big_eval_t<LL>(fd, params, bb, ebuf, gbuf, chi_part, se_part, st);
+        return big_model_t<LL>(fd, params, bb, ebuf, chi_part, se_part, st);
         SR_BG_SIZES(SR_BG_E)
 #undef SR_BG_E
+        default:
+            return 0;
+    }
+}
+
+int launch_big_window(const FieldDev &fd, const float *params, const float *ebuf, float *gbuf, cudaStream_t st) {
+    if (fd.M <= 0) return 0;
+    big_window_adj_kernel<<<fd.E * fd.M * fd.f * fd.f, kWinThreads, fft_big_window_smem(fd.Tk, fd.f), st>>>(fd, params,
+                                                                                                       ebuf, gbuf);
+    return 1;
+}
+
+int launch_big_adj(const FieldDev &fd, const BigBuffers &bb, cudaStream_t st) {
+    switch (fd.fft_L) {
+#define SR_BG_A(LL) \
+    case LL:        \
+        return big_adj_t<LL>(fd, bb, st);
+        SR_BG_SIZES(SR_BG_A)
+#undef SR_BG_A
         default:
             return 0;
     }

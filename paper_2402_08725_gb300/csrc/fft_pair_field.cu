@@ -235,7 +235,8 @@ __device__ __noinline__ void hhat_pair(const FieldDev &fd, const float *__restri
     const bool hasb = pb < nph;
     const int pay = pa / f, pax = pa - pay * f, pby = pb / f, pbx = pb - pby * f;
     const float *h = params + fd.param_off;
-    for (int t = threadIdx.x; t < N * N; t += blockDim.x) {
+#pragma unroll 8
+    for (int t = threadIdx.x; t < N * N; t += blockDim.x) {  // eight pixels' loads together
         const int y = t / N, x = t - y * N;
         const float va = h[(long long)(f * y + pay) * F + f * x + pax];
         const float vb = hasb ? h[(long long)(f * y + pby) * F + f * x + pbx] : 0.f;
@@ -359,6 +360,7 @@ __device__ __noinline__ void hgrad_pair(const FieldDev &fd, const float2 *__rest
     const int pay = pa / f, pax = pa - pay * f, pby = pb / f, pbx = pb - pby * f;
     const float *T0 = fd.starlet + (long long)fd.J * F * F;
     float *gh = grad + fd.param_off;
+#pragma unroll 8
     for (int t = threadIdx.x; t < N * N; t += blockDim.x) {
         const int y = t / N, x = t - y * N;
         const float2 v = Z[y * P + pcol<L>(x)];

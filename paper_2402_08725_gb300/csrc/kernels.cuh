@@ -31,7 +31,8 @@ void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, const f
                         float *hs, cudaStream_t st);
 // pts_fields / l1_pts / pts_g: the point-source prior's table and outputs (launch_pts_prior), or
 // nullptr when no field of the table has the term
-void launch_finalize(const FieldDev *fields, int n_fields, const double *chi_part, const double *se_part,
+// Returns its launches.
+int launch_finalize(const FieldDev *fields, int n_fields, const double *chi_part, const double *se_part,
                      const double *l1_part, const float *ps_da, const float *ps_du, float *grad, double *losses,
                      double *total, cudaStream_t st, const FieldDev *pts_fields = nullptr,
                      const double *l1_pts = nullptr, const float *pts_g = nullptr, const float *hs = nullptr);
@@ -79,10 +80,12 @@ sr_status configure_fft_big(int optin);
 // kernel spectra [E][f^2][L/2+1][L] (transposed half spectra) at fd.fft_khat, with scratch zb, zt of
 // E * pairs * Tk * L complex each
 int launch_big_kappa(const FieldDev &fd, float2 *zb, float2 *zt, cudaStream_t st);
-// the model, residual, chi^2 / sum e partial sums (n_tiles = N slots per epoch), the adjoint spectra
-// and the source windows' adjoint images (gbuf); returns the number of launches
-int launch_big_eval(const FieldDev &fd, const float *params, const BigBuffers &bb, float *ebuf, float *gbuf,
-                    double *chi_part, double *se_part, cudaStream_t st);
+// the model, residual and chi^2 / sum e partial sums (n_tiles = N slots per epoch); then, in any order,
+// the source windows' adjoint images (gbuf) and the adjoint spectra.  Each returns its launches.
+int launch_big_model(const FieldDev &fd, const float *params, const BigBuffers &bb, float *ebuf, double *chi_part,
+                     double *se_part, cudaStream_t st);
+int launch_big_window(const FieldDev &fd, const float *params, const float *ebuf, float *gbuf, cudaStream_t st);
+int launch_big_adj(const FieldDev &fd, const BigBuffers &bb, cudaStream_t st);
 // dL/dh of the field (after the starlet kernels, whose gradient it adds)
 int launch_big_hgrad(const FieldDev &fd, const BigBuffers &bb, float *grad, cudaStream_t st);
 
@@ -117,6 +120,8 @@ void launch_host_copy(const float *src, float *dst, long long n, const double *t
 constexpr int kStarletMapBit = 16;
 // bits of forms that shorten the comb-band blocks to 4 or 8 rows (starlet_comb_rows_bits)
 constexpr int kStarletRows4 = 32, kStarletRows8 = 64;
+// ... and run the comb-band fields of grids up to 256 pixels as clusters, one launch for all levels
+constexpr int kStarletClusterBit = 128;
 int starlet_field_form(int F, int J);
 int starlet_comb_rows_of(int forms);
 int starlet_comb_rows_bits(const int *F, const int *J, int n, int n_sms);

@@ -234,8 +234,7 @@ int launch_plain_eval(const FieldDev *fields, const FieldDev &hf, const float *s
     n += launch_starlet(fields, 1, hf.F, forms, chunks, n_chunks, hf.J, params, l1_part, st);
     plain_hgrad_kernel<<<gF, 256, 0, st>>>(fields, pb.gsum, grad);
     ++n;
-    launch_finalize(fields, 1, chi_part, se_part, l1_part, ps_da, ps_du, grad, losses, total, st);
-    n += 2;
+    n += launch_finalize(fields, 1, chi_part, se_part, l1_part, ps_da, ps_du, grad, losses, total, st);
     return n;
 }
 

@@ -30,7 +30,8 @@ __device__ __forceinline__ double strided_sum4(const double *__restrict__ v, lon
 }
 
 // Deterministic block sum of two doubles (fixed shuffle tree, warps summed in order).
-__device__ __forceinline__ void block_sum2(double &a, double &b, double (*red)[kThreads / 32]) {
+template <int NW>
+__device__ __forceinline__ void block_sum2(double &a, double &b, double (*red)[NW]) {
     a = warp_sum(a);
     b = warp_sum(b);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;

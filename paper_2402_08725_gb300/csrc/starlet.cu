@@ -11,7 +11,10 @@
 // Scratch per field (planes of F*F floats): c_1..c_{J-1} (planes 0..J-2), a spare plane (J-1),
 // and two T planes (J, J+1) used alternately; T_0 ends in plane J.
 //
-// Three ways to run a level, chosen per field (starlet_form):
+// Four ways to run, chosen per field (starlet_form) and table:
+//  * clusters (grids up to 256 pixels in tables too small to fill the GPU): all levels of a field in
+//    one launch, on a cluster of 8 blocks that take the comb bands below, with a cluster barrier
+//    between levels instead of a launch (see starlet_cluster_kernel).
 //  * comb bands (most fields): the rows rho, rho + s, rho + 2 s, ... of level j (step s = 2^j)
 //    are one column tap apart, so a block taking 16 consecutive rows of one such comb stages
 //    only 20 input rows at any level; otherwise the same as the bands below, whose arithmetic
@@ -56,6 +59,7 @@ constexpr int kTileSmemBytes = 160 * 1024;     // shared memory of a tile block 
 // consecutive rows of one comb and stages 20 (two more on each side) instead of 16 + 4 s.
 constexpr int kCombRows = 16;  // rows of a comb per block (fewer for small tables, see comb_rows)
 constexpr int kCombMaxF = kBandSmemBytes / ((2 * kCombRows + 4) * (int)sizeof(float));  // adjoint budget
+constexpr int kCombFwdSmemBytes = 2 * (kCombRows + 4) * kCombMaxF * (int)sizeof(float);  // staged and filtered rows
 // Blocks of level j: s combs of ceil(ceil(F / s) / cr) chunks each.
 __host__ __device__ inline int comb_chunks(int F, int s, int cr = kCombRows) {
     return ((F + s - 1) / s + cr - 1) / cr;
@@ -89,6 +93,12 @@ __host__ __device__ inline bool starlet_tiled(int F, int J) {
         if ((long long)(1 << j) * comb_chunks(F, 1 << j, kCombGroup) * nbx > slots) return false;
     return true;
 }
+
+// Widest grid that runs as a cluster, its blocks (eight is the largest portable cluster) and threads.
+// A block takes one comb chunk of a level, of as many rows (a multiple of 4) as that needs.
+constexpr int kClusterMaxF = 256, kClusterBlocks = 8, kClusterThreads = 1024;
+__host__ __device__ inline int cluster_rows(int F) { return 4 * ((F + 4 * kClusterBlocks - 1) / (4 * kClusterBlocks)); }
+constexpr int kClusterMaxRows = 4 * ((kClusterMaxF + 4 * kClusterBlocks - 1) / (4 * kClusterBlocks));
 
 // 0 bands, 1 tiles, 3 comb bands; 2: none (no shape of at most 8 scales on a grid of at most
 // 32768 pixels comes here; sr_create_problem rejects one that would)
@@ -266,30 +276,46 @@ starlet_band_adj_kernel(const FieldDev *__restrict__ fields, const float *__rest
     }
 }
 
+// A row of F floats into shared memory by one warp, eight loads of a lane in flight together: the
+// planes come from L2 (600 cycles and more away), and a level of a small grid is little else.
+__device__ __forceinline__ void stage_row(float *dst, const float *src, int F, int lane) {
+    int x = lane;
+    for (; x + 224 < F; x += 256) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = src[x + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) dst[x + 32 * u] = v[u];
+    }
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = x + 32 * u < F ? src[x + 32 * u] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (x + 32 * u < F) dst[x + 32 * u] = v[u];
+}
+
 // Forward level j as comb bands: block b takes rows y_t = rho + s (k0 + t), t < cr, of comb rho,
-// filters rows rho + s (k0 - 2 + i), i < cr + 4 (mirrored), along x into shared memory, then along
-// y: each output row's five taps are staged rows t .. t + 4.  The same values, in the same order,
-// as the bands.  Block (b, field), b = rho * nk + k0 / cr.
+// stages rows rho + s (k0 - 2 + i), i < cr + 4 (mirrored), filters them along x, then along y: each
+// output row's five taps are staged rows t .. t + 4.  The same values, in the same order,
+// as the bands.  b = rho * nk + k0 / cr.
 template <bool MAP>
-__global__ void __launch_bounds__(256)
-starlet_comb_fwd_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params,
-                        double *__restrict__ l1_part, int j, int cr) {
-    extern __shared__ float sb[];
-    __shared__ float2 s_row[kCombRows];
-    const FieldDev &fd = fields[blockIdx.y];
-    const int F = fd.F, J = fd.J;
-    if (j > J - 2 || starlet_form(F, J) != 3) return;
-    const int s = 1 << j, nk = comb_chunks(F, s, cr), b = blockIdx.x;
-    if (b >= s * nk) return;
+__device__ __forceinline__ void comb_fwd_block(const FieldDev &fd, const float *params, double *l1_part, int j, int cr,
+                                               int b, float *sb, float2 *s_row) {
+    const int F = fd.F, s = 1 << j, nk = comb_chunks(F, s, cr);
     const int rho = b / nk, k0 = (b - rho * nk) * cr;
     const int Tr = max(0, min(cr, (F - rho + s - 1) / s - k0));  // rows of the comb in the grid
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const float *cj = c_plane(fd, params, j);
     const float *wm1 = MAP ? wmap_plane(fd, j) : nullptr;
     const int R = Tr > 0 ? Tr + 4 : 0;
+    float *raw = sb, *fil = sb + (long long)(cr + 4) * F;
+    for (int i = warp; i < R; i += nwarp)
+        stage_row(raw + (long long)i * F, cj + (long long)mirror_at(rho + s * (k0 - 2 + i), F) * F, F, lane);
+    __syncthreads();
     for (int i = warp; i < R; i += nwarp) {
-        const float *row = cj + (long long)mirror_at(rho + s * (k0 - 2 + i), F) * F;
-        float *dst = sb + (long long)i * F;
+        const float *row = raw + (long long)i * F;
+        float *dst = fil + (long long)i * F;
         for (int x = lane; x < F; x += 32) {
             float acc = 0.f;
             if (x >= 2 * s && x <= F - 1 - 2 * s) {  // all taps inside: no mirror
@@ -306,13 +332,14 @@ starlet_comb_fwd_kernel(const FieldDev *__restrict__ fields, const float *__rest
     float *cn = fd.starlet + (long long)j * F * F;  // c_{j+1}
     for (int t = warp; t < Tr; t += nwarp) {
         const long long ro = (long long)(rho + s * (k0 + t)) * F;
+        const float *mid = raw + (long long)(t + 2) * F;  // c_j of the row
         float l1_row = 0.f;
         for (int x = lane; x < F; x += 32) {
             float acc = 0.f;
 #pragma unroll
-            for (int m = -2; m <= 2; ++m) acc += kB3[m + 2] * sb[(long long)(t + 2 + m) * F + x];
+            for (int m = -2; m <= 2; ++m) acc += kB3[m + 2] * fil[(long long)(t + 2 + m) * F + x];
             cn[ro + x] = acc;
-            l1_row += fabsf(cj[ro + x] - acc) * wmap_w(wm1, ro + x);
+            l1_row += fabsf(mid[x] - acc) * wmap_w(wm1, ro + x);
         }
         const FSum r = fsum_warp(FSum{l1_row, 0.f});  // the row's sum (lanes in a fixed tree)
         if (lane == 0) s_row[t] = make_float2(r.hi, r.lo);
@@ -338,14 +365,8 @@ starlet_comb_fwd_kernel(const FieldDev *__restrict__ fields, const float *__rest
 // preimages (rows within 2 s of the grid's edges, in other combs) are read from the plane.  The
 // same values, in the same order, as the bands.
 template <bool MAP>
-__global__ void __launch_bounds__(256, 4)  // at most 64 registers: four blocks per SM
-starlet_comb_adj_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params, int j, int cr) {
-    extern __shared__ float sb[];
-    const FieldDev &fd = fields[blockIdx.y];
-    const int F = fd.F, J = fd.J;
-    if (j > J - 2 || starlet_form(F, J) != 3) return;
-    const int s = 1 << j, nk = comb_chunks(F, s, cr), b = blockIdx.x;
-    if (b >= s * nk) return;
+__device__ __forceinline__ void comb_adj_block(const FieldDev &fd, const float *params, int j, int cr, int b, float *sb) {
+    const int F = fd.F, J = fd.J, s = 1 << j, nk = comb_chunks(F, s, cr);
     const int rho = b / nk, k0 = (b - rho * nk) * cr;
     const int Tr = max(0, min(cr, (F - rho + s - 1) / s - k0));
     if (Tr == 0) return;
@@ -364,7 +385,19 @@ starlet_comb_adj_kernel(const FieldDev *__restrict__ fields, const float *__rest
     for (int i = warp; i < Tr + 4; i += nwarp) {
         const int r = rho + s * (k0 - 2 + i);
         if (r < 0 || r >= F) continue;  // never read: the gather tests the same range
-        for (int x = lane; x < F; x += 32) vb[(long long)i * F + x] = vval(r, x);
+        float *dst = vb + (long long)i * F;
+        if (!top) {
+            stage_row(dst, Vn + (long long)r * F, F, lane);
+            continue;
+        }
+        for (int x0 = lane; x0 < F; x0 += 128) {  // four pixels' loads together
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = x0 + 32 * u < F ? vval(r, x0 + 32 * u) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (x0 + 32 * u < F) dst[x0 + 32 * u] = v[u];
+        }
     }
     __syncthreads();
     for (int t = warp; t < Tr; t += nwarp) {
@@ -398,11 +431,88 @@ starlet_comb_adj_kernel(const FieldDev *__restrict__ fields, const float *__rest
     for (int t = warp; t < Tr; t += nwarp) {
         const long long ro = (long long)(rho + s * (k0 + t)) * F;
         const float *trow = tb + (long long)t * F;
-        for (int x = lane; x < F; x += 32) {
-            const float acc = adj_1d(trow, x, F, s, 1);
-            const float tj = gamma_of(cj[ro + x] - cn[ro + x], lw1 * wmap_w(wm1, ro + x)) + acc;
-            out[ro + x] = j >= 1 ? tj - gamma_of(cjm[ro + x] - cj[ro + x], lw0 * wmap_w(wm0, ro + x)) : tj;
+        for (int x0 = lane; x0 < F; x0 += 128) {  // four pixels' loads together
+            float c0[4], c1[4], cm[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int x = x0 + 32 * u;
+                const bool in = x < F;
+                c0[u] = in ? cj[ro + x] : 0.f;
+                c1[u] = in ? cn[ro + x] : 0.f;
+                cm[u] = in ? cjm[ro + x] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int x = x0 + 32 * u;
+                if (x >= F) continue;
+                const float acc = adj_1d(trow, x, F, s, 1);
+                const float tj = gamma_of(c0[u] - c1[u], lw1 * wmap_w(wm1, ro + x)) + acc;
+                out[ro + x] = j >= 1 ? tj - gamma_of(cm[u] - c0[u], lw0 * wmap_w(wm0, ro + x)) : tj;
+            }
         }
+    }
+}
+
+// One level of the fields wider than `above`, one launch: block (b, field).
+template <bool MAP>
+__global__ void __launch_bounds__(256)
+starlet_comb_fwd_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params,
+                        double *__restrict__ l1_part, int j, int cr, int above) {
+    extern __shared__ float sb[];
+    __shared__ float2 s_row[kCombRows];
+    const FieldDev &fd = fields[blockIdx.y];
+    if (j > fd.J - 2 || starlet_form(fd.F, fd.J) != 3 || fd.F <= above) return;
+    if ((int)blockIdx.x >= (1 << j) * comb_chunks(fd.F, 1 << j, cr)) return;
+    comb_fwd_block<MAP>(fd, params, l1_part, j, cr, blockIdx.x, sb, s_row);
+}
+
+template <bool MAP>
+__global__ void __launch_bounds__(256, 4)  // at most 64 registers: four blocks per SM
+starlet_comb_adj_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params, int j, int cr, int above) {
+    extern __shared__ float sb[];
+    const FieldDev &fd = fields[blockIdx.y];
+    if (j > fd.J - 2 || starlet_form(fd.F, fd.J) != 3 || fd.F <= above) return;
+    if ((int)blockIdx.x >= (1 << j) * comb_chunks(fd.F, 1 << j, cr)) return;
+    comb_adj_block<MAP>(fd, params, j, cr, blockIdx.x, sb);
+}
+
+// Every thread of the cluster arrives and waits; writes before it (global ones included) are visible
+// to the cluster's reads after it.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// All levels, forward and adjoint, of a field on one cluster of kClusterBlocks blocks: the comb blocks
+// of a level are dealt over the cluster, and a cluster barrier stands where a launch ends.  The planes
+// stay in L2.  A level of a small grid is a chain of a few staged rows, so its launch (about 4 us with
+// its ramp, up to 14 of them in a row) costs more than its work: PSF fit of 16 stars on 128 x 128, J = 5
+// 129 -> 80 us with the shorter finalize, fit on 135 x 135 with both priors 211 -> 100 us.  A table whose
+// levels fill the GPU runs them level by level, with less halo per block and no block waiting at a
+// barrier: 256 fields 10.17 ms an evaluation that way, 10.53 in clusters.  Grid (kClusterBlocks, fields).
+template <bool MAP>
+__global__ void __launch_bounds__(kClusterThreads)
+starlet_cluster_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params, double *l1_part) {
+    extern __shared__ float sb[];
+    __shared__ float2 s_row[kClusterMaxRows];
+    const FieldDev &fd = fields[blockIdx.y];
+    const int F = fd.F, J = fd.J;
+    if (starlet_form(F, J) != 3 || F > kClusterMaxF) return;  // the whole cluster
+    const int cr = cluster_rows(F);
+    for (int j = 0; j <= J - 2; ++j) {
+        const int nb = (1 << j) * comb_chunks(F, 1 << j, cr);
+        for (int b = blockIdx.x; b < nb; b += kClusterBlocks) {
+            comb_fwd_block<MAP>(fd, params, l1_part, j, cr, b, sb, s_row);
+            __syncthreads();
+        }
+        cluster_sync();
+    }
+    for (int j = J - 2; j >= 0; --j) {
+        const int nb = (1 << j) * comb_chunks(F, 1 << j, cr);
+        for (int b = blockIdx.x; b < nb; b += kClusterBlocks) {
+            comb_adj_block<MAP>(fd, params, j, cr, b, sb);
+            __syncthreads();
+        }
+        if (j > 0) cluster_sync();
     }
 }
 
@@ -572,15 +682,15 @@ int starlet_forms_single(int F, int J, bool map) {
 
 int starlet_comb_rows_of(int forms) { return (forms & kStarletRows8) ? 8 : (forms & kStarletRows4) ? 4 : kCombRows; }
 
-// Rows per comb block for a table of comb-band fields (F, J of each): 16, or 8 or 4 when the
-// table's level-0 blocks would not fill twice the SMs.  The results do not depend on it (the
+// Rows per comb block for a table of comb-band fields (F, J of each): 16, or 8 or 4, and clusters, when
+// the table's level-0 blocks would not fill twice the SMs.  The results do not depend on it (the
 // prior's partial sums are kept per 4-row group).  Returns the forms bit to add (0 for 16 rows).
 int starlet_comb_rows_bits(const int *F, const int *J, int n, int n_sms) {
     long long blocks = 0;
     for (int i = 0; i < n; ++i)
         if (starlet_form(F[i], J[i]) == 3) blocks += comb_chunks(F[i], 1);
     if (blocks == 0 || blocks >= 2LL * n_sms) return 0;
-    return 2 * blocks >= 2LL * n_sms ? kStarletRows8 : kStarletRows4;
+    return (2 * blocks >= 2LL * n_sms ? kStarletRows8 : kStarletRows4) | kStarletClusterBit;
 }
 
 int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, const ChunkItem *chunks,
@@ -595,19 +705,26 @@ int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, co
         cudaFuncSetAttribute(starlet_band_adj_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
         cudaFuncSetAttribute(starlet_tile_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes);
         cudaFuncSetAttribute(starlet_tile_adj_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes);
-        cudaFuncSetAttribute(starlet_comb_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
+        cudaFuncSetAttribute(starlet_comb_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombFwdSmemBytes);
         cudaFuncSetAttribute(starlet_comb_adj_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
-        cudaFuncSetAttribute(starlet_comb_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
+        cudaFuncSetAttribute(starlet_comb_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombFwdSmemBytes);
         cudaFuncSetAttribute(starlet_comb_adj_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
+        cudaFuncSetAttribute(starlet_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
+        cudaFuncSetAttribute(starlet_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
     });
     const bool bands = (forms & 1) != 0, tiles = (forms & 2) != 0;
-    const bool combs = (forms & 8) != 0, map = (forms & kStarletMapBit) != 0;
-    // comb bands: s combs of comb_chunks blocks at level j; staging of cr + 4 (forward) or
+    const bool map = (forms & kStarletMapBit) != 0;
+    // comb-band fields: in clusters up to kClusterMaxF when the table asks for it, the others (if any)
+    // level by level
+    const bool clusters = (forms & 8) != 0 && (forms & kStarletClusterBit) != 0;
+    const int above = clusters ? kClusterMaxF : 0;
+    const bool combs = (forms & 8) != 0 && Fmax > above;
+    // comb bands: s combs of comb_chunks blocks at level j; staging of 2 (cr + 4) (forward) or
     // 2 cr + 4 (adjoint) rows of the widest comb-band grid
     const int cr = starlet_comb_rows_of(forms);
     const int Fc = std::min(Fmax, kCombMaxF);
     auto cgrid = [&](int j) { return dim3((unsigned)((1 << j) * comb_chunks(Fc, 1 << j, cr)), n_fields); };
-    const int comb_fwd_smem = (cr + 4) * Fc * (int)sizeof(float);
+    const int comb_fwd_smem = 2 * (cr + 4) * Fc * (int)sizeof(float);
     const int comb_adj_smem = (2 * cr + 4) * Fc * (int)sizeof(float);
     auto tgrid = [&](int j) {
         const int sj = 1 << j;
@@ -617,6 +734,22 @@ int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, co
         return (int)std::min<long long>(floats * (long long)sizeof(float), kTileSmemBytes);
     };
     int n = 0;
+    if (clusters) {
+        const int Fk = std::min(Fmax, kClusterMaxF), rk = cluster_rows(Fk);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kClusterBlocks;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kClusterBlocks, n_fields);
+        cfg.blockDim = dim3(kClusterThreads);
+        cfg.dynamicSmemBytes = 2 * (rk + 4) * Fk * sizeof(float);
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, map ? starlet_cluster_kernel<true> : starlet_cluster_kernel<false>, fields, params, l1_part);
+        ++n;
+    }
     const dim3 bgrid((Fmax + kBandRows - 1) / kBandRows, n_fields);
     // shared memory of level j: (2 * 16 + 4 * 2^j) rows of the widest grid, at most the budget
     // (which every banded field's deepest level fits, so its shallower levels fit too)
@@ -634,9 +767,9 @@ int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, co
         }
         if (combs) {
             if (map)
-                starlet_comb_fwd_kernel<true><<<cgrid(j), 256, comb_fwd_smem, st>>>(fields, params, l1_part, j, cr);
+                starlet_comb_fwd_kernel<true><<<cgrid(j), 256, comb_fwd_smem, st>>>(fields, params, l1_part, j, cr, above);
             else
-                starlet_comb_fwd_kernel<false><<<cgrid(j), 256, comb_fwd_smem, st>>>(fields, params, l1_part, j, cr);
+                starlet_comb_fwd_kernel<false><<<cgrid(j), 256, comb_fwd_smem, st>>>(fields, params, l1_part, j, cr, above);
             ++n;
         }
         if (tiles) {
@@ -658,9 +791,9 @@ int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, co
         }
         if (combs) {
             if (map)
-                starlet_comb_adj_kernel<true><<<cgrid(j), 256, comb_adj_smem, st>>>(fields, params, j, cr);
+                starlet_comb_adj_kernel<true><<<cgrid(j), 256, comb_adj_smem, st>>>(fields, params, j, cr, above);
             else
-                starlet_comb_adj_kernel<false><<<cgrid(j), 256, comb_adj_smem, st>>>(fields, params, j, cr);
+                starlet_comb_adj_kernel<false><<<cgrid(j), 256, comb_adj_smem, st>>>(fields, params, j, cr, above);
             ++n;
         }
         if (tiles) {
