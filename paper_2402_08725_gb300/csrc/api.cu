@@ -267,8 +267,8 @@ struct Plan {
     int prof_count = 0;
     std::vector<cudaEvent_t> prof_ev;
     // Branches of the evaluation beside its own stream (see Branch): the starlet prior on h, the
-    // point-source prior, and the sources' gradients
-    Branch prior, pts, src;
+    // point-source prior, the sources' gradients, and an optimiser step's counter
+    Branch prior, pts, src, step;
     DevArena arena;
     ~Plan() {
         if (graph) cudaGraphExecDestroy(graph);
@@ -1131,6 +1131,7 @@ static sr_status ensure_opt_buffers(Plan *pl) {
     if ((st = pl->arena.alloc(&pl->opt_m, pl->n_params)) != SR_OK) return st;
     if ((st = pl->arena.alloc(&pl->opt_v, pl->n_params)) != SR_OK) return st;
     if ((st = pl->arena.alloc(&pl->grad_int, pl->n_params)) != SR_OK) return st;
+    if (!pl->plain && (st = pl->step.open()) != SR_OK) return st;
     SR_CUDA(cudaMemset(pl->opt_m, 0, sizeof(float) * pl->n_params));
     SR_CUDA(cudaMemset(pl->opt_v, 0, sizeof(float) * pl->n_params));
     SR_CUDA(cudaMemset(pl->d_t, 0, sizeof(long long)));
@@ -1163,14 +1164,6 @@ static OptimArgs optim_args(const Plan *pl, const sr_optim_cfg &c) {
     return a;
 }
 
-__global__ void record_loss_kernel(const double *total, double *const *hist_ptr, const long long *t,
-                                   const long long *base) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double *h = *hist_ptr;
-        if (h) h[*t - *base] = *total;
-    }
-}
-
 // n optimiser steps on plan `pl` (eager when the stream cannot be captured).
 static sr_status run_steps(Plan *pl, cudaStream_t st, float *params, int n_steps, const sr_optim_cfg *cfg,
                            double *losses_dev, const std::vector<const float *> *s_raw) {
@@ -1180,10 +1173,12 @@ static sr_status run_steps(Plan *pl, cudaStream_t st, float *params, int n_steps
     SR_CUDA(cudaMemcpyAsync(pl->d_hist_ptr, &losses_dev, sizeof(double *), cudaMemcpyHostToDevice, st));
     SR_CUDA(cudaMemcpyAsync(pl->d_hist_base, pl->d_t, sizeof(long long), cudaMemcpyDeviceToDevice, st));
     auto enqueue_one = [&](cudaStream_t s2) {
+        cudaStream_t pro = pl->step.fork(s2);
+        launch_opt_prologue(oa, pl->d_t, pl->d_bc, pro);
         pl->launches = run_eval(pl, params, pl->grad_int, s2, s_raw);
-        record_loss_kernel<<<1, 32, 0, s2>>>(pl->total, pl->d_hist_ptr, pl->d_t, pl->d_hist_base);
-        launch_opt_step((long long)pl->n_params, params, pl->grad_int, pl->opt_m, pl->opt_v, pl->d_group, oa, pl->d_t,
-                        pl->d_bc, s2);
+        pl->step.join(pro, s2);
+        launch_opt_update((long long)pl->n_params, params, pl->grad_int, pl->opt_m, pl->opt_v, pl->d_group, oa, pl->d_t,
+                          pl->d_bc, pl->total, pl->d_hist_ptr, pl->d_hist_base, s2);
     };
     // the host copy of losses_dev must outlive the async copy above
     SR_CUDA(cudaStreamSynchronize(st));

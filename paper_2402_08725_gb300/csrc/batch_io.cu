@@ -96,9 +96,10 @@ __global__ void bio_kappa_kernel(const BioEntry *__restrict__ tab, const long lo
          i += (long long)gridDim.x * blockDim.x) {
         const int e = entry_of(off, n, i);
         const BioEntry &b = tab[e];
-        const long long local = i - off[e], per = (long long)b.f * b.f * b.Tk * b.Tk;
-        const long long ep = local / per;
-        b.kappa[local] = kappa_fold(b.s + ep * b.K * b.K, b.K, b.f, b.Tk, b.tau_lo, local - ep * per);
+        const long long local = i - off[e];
+        const int per = b.f * b.f * b.Tk * b.Tk;
+        const long long ep = local < (1LL << 31) ? (int)local / per : local / per;
+        b.kappa[local] = kappa_fold(b.s + ep * b.K * b.K, b.K, b.f, b.Tk, b.tau_lo, (int)(local - ep * per));
     }
 }
 

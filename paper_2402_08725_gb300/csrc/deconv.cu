@@ -42,7 +42,7 @@ __global__ void kappa_prep_kernel(const float *__restrict__ s, float *__restrict
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         const long long i = idx / per;
-        kappa[idx] = kappa_fold(s + i * K * K, K, f, Tk, tau_lo, idx - i * per);
+        kappa[idx] = kappa_fold(s + i * K * K, K, f, Tk, tau_lo, (int)(idx - i * per));
     }
 }
 
@@ -624,8 +624,17 @@ finalize_kernel(const FieldDev *__restrict__ fields, const double *__restrict__ 
                     const double gx = ps_du[b], gy = ps_du[b + 1];
                     acc += ax == 0 ? (double)r.x * gx + (double)r.y * gy : -(double)r.y * gx + (double)r.x * gy;
                 }
-            } else {
-                for (int i = lane; i < E; i += 32) acc += (double)ps_du[2 * (fd.ps_slot + (long long)i * M + k) + ax];
+            } else {  // four interleaved sums per lane, their loads in flight together
+                double p[4] = {0.0, 0.0, 0.0, 0.0};
+                const float *pu = ps_du + 2 * (fd.ps_slot + k) + ax;
+                for (int i = lane; i < E; i += 128) {
+                    float v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[u] = i + 32 * u < E ? pu[2 * (long long)(i + 32 * u) * M] : 0.f;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) p[u] += (double)v[u];
+                }
+                acc = (p[0] + p[1]) + (p[2] + p[3]);
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);

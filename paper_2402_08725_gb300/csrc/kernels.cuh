@@ -180,8 +180,12 @@ struct OptimArgs {
     float lr[SR_MAX_GROUPS];
     float lo[SR_MAX_GROUPS];
 };
-void launch_opt_step(long long n, float *params, const float *grad, float *m, float *v, const uint8_t *group,
-                     const OptimArgs &a, long long *t_dev, float *bc_dev, cudaStream_t st);
+// the step counter's increment and the step's bias corrections
+void launch_opt_prologue(const OptimArgs &a, long long *t_dev, float *bc_dev, cudaStream_t st);
+// the update, after both; *total goes to (*hist)[*t_dev - 1 - *hist_base] unless *hist is NULL
+void launch_opt_update(long long n, float *params, const float *grad, float *m, float *v, const uint8_t *group,
+                       const OptimArgs &a, const long long *t_dev, const float *bc_dev, const double *total,
+                       double *const *hist, const long long *hist_base, cudaStream_t st);
 
 // --- input preparation (prep.cu) ---
 void launch_inv_var(const float *sigma, float *w, long long n, int *bad_flag, cudaStream_t st);
