@@ -225,7 +225,7 @@ struct Plan {
     int Fmax = 0;               // widest fine grid of the table (the starlet band grid)
     int starlet_forms = 0;  // 1 << starlet_field_form of every field (bands, tiles, comb bands)
     float *ebuf = nullptr, *gbuf = nullptr, *ps_da = nullptr, *ps_du = nullptr;
-    double *chi_part = nullptr, *se_part = nullptr, *l1_part = nullptr, *losses = nullptr, *total = nullptr;
+    double *chi_part = nullptr, *se_part = nullptr, *l1_part = nullptr, *l1_sum = nullptr, *losses = nullptr, *total = nullptr;
     // frequency-domain form
     int n_fft_items = 0, n_fft_fields = 0, max_pairs = 1, smem_fft = 0, smem_fx = 0, grid_fft = 0;
     int max_acc_points = 0;  // largest f^2 L (L/2 + 1) of the transform fields
@@ -822,6 +822,9 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
     if ((st = A.alloc(&pl->ps_da, n_ps_slots)) != SR_OK) return st;
     if ((st = A.alloc(&pl->ps_du, 2 * n_ps_slots)) != SR_OK) return st;
     if ((st = A.alloc(&pl->l1_part, (size_t)l1slot)) != SR_OK) return st;
+    for (const FieldDev &fd : pl->h_fields)
+        if (pl->kind == SR_DECONV && !pl->l1_sum && (long long)(fd.J - 1) * fd.n_chunks > kL1Many)
+            if ((st = A.alloc(&pl->l1_sum, (size_t)n * kL1Blocks)) != SR_OK) return st;
     if ((st = A.alloc(&pl->losses, (size_t)n)) != SR_OK) return st;
     if (hs_len > 0 && (st = A.alloc(&pl->hs, (size_t)hs_len)) != SR_OK) return st;
     if ((st = A.alloc(&pl->total, 1)) != SR_OK) return st;
@@ -952,6 +955,10 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
     auto launch_priors = [&]() {
         n += launch_starlet(pl->d_fields, pl->n_fields, pl->Fmax, pl->starlet_forms, pl->d_chunks, pl->n_chunks,
                             pl->Jmax, params, pl->l1_part, prior);
+        if (pl->l1_sum) {
+            launch_l1_sum(pl->d_fields, pl->n_fields, pl->l1_part, pl->l1_sum, prior);
+            ++n;
+        }
         if (pl->n_sh > 0)
             n += launch_pts_prior(pl->d_sh, pl->d_fields, pl->n_sh, pl->sh_Fmax, pl->sh_Mmax, pl->sh_starlet_forms,
                                   pl->d_sh_chunks, pl->n_sh_chunks, pl->sh_Jmax, params, pl->abar, pl->pbar, pl->l1_pts,
@@ -1019,7 +1026,7 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
     pl->pts.join(pts, st);
     pl->src.join(src, st);
     n += launch_finalize(pl->d_fields, pl->n_fields, pl->chi_part, pl->se_part, pl->l1_part, pl->ps_da, pl->ps_du, grad,
-                    pl->losses, pl->total, st, pl->n_sh > 0 ? pl->d_sh : nullptr, pl->l1_pts, pl->pts_g, pl->hs);
+                    pl->losses, pl->total, st, pl->n_sh > 0 ? pl->d_sh : nullptr, pl->l1_pts, pl->pts_g, pl->hs, pl->l1_sum);
     return n;
 }
 

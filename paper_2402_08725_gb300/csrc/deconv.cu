@@ -577,6 +577,21 @@ hshift_grad_kernel(const FieldDev *__restrict__ fields, const float *__restrict_
     }
 }
 
+// The prior's partial sums of a field with more than kL1Many of them (wide grids: 46 080 at 1536 x 1536,
+// J = 6) in kL1Blocks sums, on the prior's branch: in the field's one finalize block they took 25 us at
+// the end of the evaluation.  Block (b, field) adds its contiguous share.
+__global__ void __launch_bounds__(kThreads)
+l1_sum_kernel(const FieldDev *__restrict__ fields, const double *__restrict__ l1_part, double *__restrict__ l1_sum) {
+    __shared__ double s_red[2][kThreads / 32];
+    const FieldDev &fd = fields[blockIdx.y];
+    const long long nl = (long long)(fd.J - 1) * fd.n_chunks;
+    if (nl <= kL1Many) return;
+    const long long lo = nl * blockIdx.x / kL1Blocks, hi = nl * (blockIdx.x + 1) / kL1Blocks;
+    double v = strided_sum4(l1_part + fd.l1_slot + lo, hi - lo), none = 0.0;
+    block_sum2(v, none, s_red);
+    if (threadIdx.x == 0) l1_sum[(long long)blockIdx.y * kL1Blocks + blockIdx.x] = v;
+}
+
 // Per-field assembly of the loss and the small parameter blocks, in fixed order.  One block per field;
 // with one field it also writes the total.  More threads do not help: the FP64 sums run at 2 additions
 // a clock per SM (37 epochs 9.8 us with 256 threads, 17.5 with 1024).
@@ -587,7 +602,7 @@ finalize_kernel(const FieldDev *__restrict__ fields, const double *__restrict__ 
                 const float *__restrict__ ps_da, const float *__restrict__ ps_du, float *__restrict__ grad,
                 double *__restrict__ losses, const FieldDev *__restrict__ pts_fields,
                 const double *__restrict__ l1_pts, const float *__restrict__ pts_g, const float *__restrict__ hs,
-                double *__restrict__ total) {
+                double *__restrict__ total, const double *__restrict__ l1_sum) {
     __shared__ double s_red[2][kFinThreads / 32];
     const FieldDev &fd = fields[blockIdx.x];
     const int E = fd.E, M = fd.M, F = fd.F, f = fd.f;
@@ -599,7 +614,8 @@ finalize_kernel(const FieldDev *__restrict__ fields, const double *__restrict__ 
     const long long nt = (long long)E * fd.n_tiles;
     const long long nl = (long long)(fd.J - 1) * fd.n_chunks;
     double chi = strided_sum4(chi_part + fd.tile_slot, nt);
-    double l1 = strided_sum4(l1_part + fd.l1_slot, nl);
+    double l1 = l1_sum && nl > kL1Many ? strided_sum4(l1_sum + (long long)blockIdx.x * kL1Blocks, kL1Blocks)
+                                       : strided_sum4(l1_part + fd.l1_slot, nl);
     if (sd) l1 += strided_sum4(l1_pts + sd->l1_slot, nl);
     block_sum2(chi, l1, s_red);
     if (threadIdx.x == 0) {
@@ -770,12 +786,16 @@ void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, const f
     hshift_grad_kernel<<<dim3(E_max, n_fields), kShiftThreads, 0, st>>>(fields, params, gbuf, hs);
 }
 
+void launch_l1_sum(const FieldDev *fields, int n_fields, const double *l1_part, double *l1_sum, cudaStream_t st) {
+    l1_sum_kernel<<<dim3(kL1Blocks, n_fields), kThreads, 0, st>>>(fields, l1_part, l1_sum);
+}
+
 int launch_finalize(const FieldDev *fields, int n_fields, const double *chi_part, const double *se_part,
                     const double *l1_part, const float *ps_da, const float *ps_du, float *grad, double *losses,
                     double *total, cudaStream_t st, const FieldDev *pts_fields, const double *l1_pts,
-                    const float *pts_g, const float *hs) {
+                    const float *pts_g, const float *hs, const double *l1_sum) {
     finalize_kernel<<<n_fields, kFinThreads, 0, st>>>(fields, chi_part, se_part, l1_part, ps_da, ps_du, grad, losses,
-                                                      pts_fields, l1_pts, pts_g, hs, total);
+                                                      pts_fields, l1_pts, pts_g, hs, total, l1_sum);
     if (n_fields == 1) return 1;
     total_kernel<<<1, 32, 0, st>>>(losses, n_fields, total);
     return 2;

@@ -35,7 +35,11 @@ void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, const f
 int launch_finalize(const FieldDev *fields, int n_fields, const double *chi_part, const double *se_part,
                      const double *l1_part, const float *ps_da, const float *ps_du, float *grad, double *losses,
                      double *total, cudaStream_t st, const FieldDev *pts_fields = nullptr,
-                     const double *l1_pts = nullptr, const float *pts_g = nullptr, const float *hs = nullptr);
+                     const double *l1_pts = nullptr, const float *pts_g = nullptr, const float *hs = nullptr, const double *l1_sum = nullptr);
+// Prior partial sums of the fields with more than kL1Many of them, pre-added into kL1Blocks each
+// (l1_sum [n_fields][kL1Blocks]; launch_finalize takes it, or nullptr to add them all itself).
+constexpr int kL1Many = 4096, kL1Blocks = 64;
+void launch_l1_sum(const FieldDev *fields, int n_fields, const double *l1_part, double *l1_sum, cudaStream_t st);
 
 // --- frequency-domain form (fft_pair.cu): in-place transforms of real image pairs ---
 bool fft_pair_size(int L);

@@ -25,8 +25,8 @@
 //    loading), so that its column pass reads one plane per tap; the signs are taken from the c
 //    planes once per output pixel.
 //  * tiles (fields too wide for comb bands of whole rows): the comb bands on 128 columns, with
-//    the 2 * 2^j halo along x (the forward reads its row taps from the c plane directly; the
-//    adjoint stages the V rows and the column-adjoint values of the tile's columns and halo,
+//    the 2 * 2^j halo along x (the forward stages the c rows, the
+//    adjoint the V rows and the column-adjoint values of the tile's columns and halo,
 //    which hold every mirror preimage its row gather reaches).
 // Fields deeper than a level skip it.
 #include <algorithm>
@@ -77,9 +77,9 @@ __host__ __device__ inline bool starlet_combed(int F, int J) {
     return true;
 }
 // Tiles (grids too wide for the comb bands): comb rows as above by 128 columns with the 2 s halo
-// along x.  Shared memory (floats) at level j: the forward's row-filtered rows (20 rows of 128),
-// the adjoint's V rows and column-adjoint rows (20 and 16 rows of 128 + 4 s).
-__host__ __device__ inline long long tile_fwd_floats(int) { return (long long)(kCombRows + 4) * kTileCols; }
+// along x.  Shared memory (floats) at level j: the forward's staged and row-filtered rows (20 rows of
+// 128 + 4 s and of 128), the adjoint's V rows and column-adjoint rows (20 and 16 rows of 128 + 4 s).
+__host__ __device__ inline long long tile_fwd_floats(int j) { return (kCombRows + 4) * (2LL * kTileCols + (4LL << j)); }
 __host__ __device__ inline long long tile_adj_floats(int j) {
     const long long s = 1LL << j;
     return (2LL * kCombRows + 4) * (kTileCols + 4 * s);
@@ -516,8 +516,7 @@ starlet_cluster_kernel(const FieldDev *__restrict__ fields, const float *__restr
     }
 }
 
-// Forward level j as tiles: the comb-band forward on the columns [x0, x0 + 128) (the row taps read
-// from c_j directly).  Block (t, field), t = (rho * nk + k0 / 16) * nbx + x0 / 128; the prior's
+// Forward level j as tiles: the comb-band forward on the columns [x0, x0 + 128) and their halo.  Block (t, field), t = (rho * nk + k0 / 16) * nbx + x0 / 128; the prior's
 // partial sums per (4-row comb group, column tile).
 template <bool MAP>
 __global__ void __launch_bounds__(256)
@@ -538,9 +537,16 @@ starlet_tile_fwd_kernel(const FieldDev *__restrict__ fields, const float *__rest
     const float *cj = c_plane(fd, params, j);
     const float *wm1 = MAP ? wmap_plane(fd, j) : nullptr;
     const int R = Tr > 0 ? Tr + 4 : 0;
+    // c_j over the tile's columns and their 2 s halo (clipped to the grid; the mirrored taps of the
+    // grid's edges lie in it), then the row filter, from shared memory
+    const int xlo = max(0, x0 - 2 * s), W = min(F, x0 + Tc + 2 * s) - xlo, WP = kTileCols + 4 * s;
+    float *raw = sb, *fil = sb + (long long)(kCombRows + 4) * WP;
+    for (int i = warp; i < R; i += nwarp)
+        stage_row(raw + (long long)i * WP, cj + (long long)mirror_at(rho + s * (k0 - 2 + i), F) * F + xlo, W, lane);
+    __syncthreads();
     for (int i = warp; i < R; i += nwarp) {
-        const float *row = cj + (long long)mirror_at(rho + s * (k0 - 2 + i), F) * F;
-        float *dst = sb + (long long)i * kTileCols;
+        const float *row = raw + (long long)i * WP - xlo;  // indexed by the grid column
+        float *dst = fil + (long long)i * kTileCols;
         for (int xx = lane; xx < Tc; xx += 32) {
             const int x = x0 + xx;
             float acc = 0.f;
@@ -558,14 +564,15 @@ starlet_tile_fwd_kernel(const FieldDev *__restrict__ fields, const float *__rest
     float *cn = fd.starlet + (long long)j * F * F;  // c_{j+1}
     for (int t = warp; t < Tr; t += nwarp) {
         const long long ro = (long long)(rho + s * (k0 + t)) * F;
+        const float *mid = raw + (long long)(t + 2) * WP - xlo;
         float l1_row = 0.f;
         for (int xx = lane; xx < Tc; xx += 32) {
             const int x = x0 + xx;
             float acc = 0.f;
 #pragma unroll
-            for (int m = -2; m <= 2; ++m) acc += kB3[m + 2] * sb[(long long)(t + 2 + m) * kTileCols + xx];
+            for (int m = -2; m <= 2; ++m) acc += kB3[m + 2] * fil[(long long)(t + 2 + m) * kTileCols + xx];
             cn[ro + x] = acc;
-            l1_row += fabsf(cj[ro + x] - acc) * wmap_w(wm1, ro + x);
+            l1_row += fabsf(mid[x] - acc) * wmap_w(wm1, ro + x);
         }
         const FSum r = fsum_warp(FSum{l1_row, 0.f});
         if (lane == 0) s_row[t] = make_float2(r.hi, r.lo);
@@ -589,7 +596,9 @@ starlet_tile_fwd_kernel(const FieldDev *__restrict__ fields, const float *__rest
 // Adjoint level j as tiles: the comb-band adjoint on the columns [x0, x0 + 128): the V rows and
 // the column-adjoint values are staged over the tile's columns and their 2 s halo (clipped to the
 // grid), which hold every mirror preimage of the row gather; the column gather's mirror
-// preimages are read from the plane.
+// preimages are read from the plane.  (Loads staged eight at a time and the last step's four pixels
+// together, as in the comb bands, are slower here, where the blocks fill the GPU: 222 -> 366 us at
+// 1536 x 1536, J = 6.)
 template <bool MAP>
 __global__ void __launch_bounds__(256)
 starlet_tile_adj_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params, int j) {
@@ -716,7 +725,7 @@ int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, co
     const bool map = (forms & kStarletMapBit) != 0;
     // comb-band fields: in clusters up to kClusterMaxF when the table asks for it, the others (if any)
     // level by level
-    const bool clusters = (forms & 8) != 0 && (forms & kStarletClusterBit) != 0;
+    const bool clusters = (forms & 8) != 0 && (forms & kStarletClusterBit) != 0 && (n_fields > 1 || Fmax <= kClusterMaxF);
     const int above = clusters ? kClusterMaxF : 0;
     const bool combs = (forms & 8) != 0 && Fmax > above;
     // comb bands: s combs of comb_chunks blocks at level j; staging of 2 (cr + 4) (forward) or
