@@ -198,7 +198,8 @@ __host__ __device__ constexpr bool prof_conj(int k2) {  // the row's values are 
 // before any is used: 9 rows of 24 bytes per thread in flight at L = 144.  (In an earlier form of this
 // pass, 8 fields of 304 epochs at L = 144: the whole phase 805 us, half of it 941, two rows kept ahead of
 // their use 1039, for loads of several ages wait for one another on a warp's six scoreboards.  Nor may
-// it spill: beside 177 KB of buffers the L1 holds a tenth of the block's spilled registers.)
+// it spill much: beside 177 KB of buffers the L1 is about 28 KB.  44 bytes are left at L = 72 and 144, 24 at
+// L = 128, for one source; 44-84 at L = 56, 72, 112, 128 and 144, 16 at L = 96, for up to four.)
 // prof_off, w_off: the profile tables and the roots of unity in pr_dyn (float2).
 template <int L, int MS>
 __device__ __noinline__ void spec_model(const FieldDev &fd, const float2 *__restrict__ hh, const float4 *__restrict__ kh,
