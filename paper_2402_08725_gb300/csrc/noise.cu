@@ -412,8 +412,8 @@ __device__ void noise_isig(const float *__restrict__ sigma, const float *__restr
 
 // Column kx of conj(Shat) / L^2 = L^-2 sum_{q,t} s[q][t] exp(2 pi i (ky (q - sh) + kx (t - sh)) / L),
 // summed over t, then over q, in FP64 and rounded once, at [position of ky][position of kx] of the
-// transforms' digit-transposed order (position R2 (k mod R1) + k / R1); kx = 0 also writes the
-// twiddles exp(-2 pi i j / L).
+// transforms' digit-transposed order (position R2 (k mod R1) + k / R1), divided by the gains of both
+// axes; kx = 0 also writes the twiddles exp(-2 pi i j / L).
 constexpr int kSpecMax = 256;
 __device__ void noise_spectrum(const float *__restrict__ s, int K, int kx, const NoiseSpec &sp, double2 *w, double2 *R) {
     const int L = sp.L, R2 = L / sp.R1;
@@ -437,7 +437,7 @@ __device__ void noise_spectrum(const float *__restrict__ s, int K, int kx, const
         R[q] = make_double2(a, b);
     }
     __syncthreads();
-    const double scale = 1.0 / ((double)L * (double)L);
+    const double scale = 1.0 / ((double)L * (double)L * sp.gain[kx]);  // and by gain[ky] below
     const int pc = R2 * (kx % sp.R1) + kx / sp.R1;
     for (int ky = threadIdx.x; ky < L; ky += blockDim.x) {
         double a = 0.0, b = 0.0;
@@ -448,7 +448,8 @@ __device__ void noise_spectrum(const float *__restrict__ s, int K, int kx, const
             j += ky;
             if (j >= L) j -= L;
         }
-        sp.S[(long long)(R2 * (ky % sp.R1) + ky / sp.R1) * L + pc] = make_float2((float)(a * scale), (float)(b * scale));
+        const double sc = scale / sp.gain[ky];
+        sp.S[(long long)(R2 * (ky % sp.R1) + ky / sp.R1) * L + pc] = make_float2((float)(a * sc), (float)(b * sc));
     }
 }
 
@@ -602,6 +603,7 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
         spec.L = fft.L;
         spec.R1 = fft.R1;
         spec.sh = fft.n == 1 ? K / 2 : 0;
+        noise_fft_gain(fft, spec.gain);
     }
     if ((rc = ws.place()) != SR_OK) return rc;
     SR_CUDA(cudaMemsetAsync(ws.base, 0, zeroed, st));  // the moments, the flag and the finishing counters

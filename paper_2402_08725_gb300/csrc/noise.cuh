@@ -9,12 +9,17 @@ namespace sr {
 struct NoiseFft {
     int L = 0, R1 = 0, n = 0, T = 0;
 };
+constexpr int kNoiseMaxL = 160;  // the largest transform
 // The kernel spectrum S [L][L] (scaled by 1 / L^2), the twiddles tw [L], and the tap offset sh: tap
-// q of s_1 acts at (q - sh) mod L.  L = 0: none.
+// q of s_1 acts at (q - sh) mod L.  gain[k]: what a transform there and back multiplies frequency k of
+// one axis by, for its roots of unity are rounded (noise_fft_gain); S is divided by it.  L = 0: none.
 struct NoiseSpec {
     float2 *S = nullptr, *tw = nullptr;
     int L = 0, R1 = 1, sh = 0;
+    double gain[kNoiseMaxL];
 };
+// gain[k], k < L, of the plan's transforms.
+void noise_fft_gain(const NoiseFft &plan, double *gain);
 // The cheapest plan (n^2 L^2) whose transforms fit smem_optin bytes of shared memory; false if none.
 bool noise_fft_plan(int F, int K, int smem_optin, NoiseFft *plan);
 // Configures the transform kernel on the current device; *resident = its blocks per SM.
