@@ -464,7 +464,7 @@ typedef struct {
     double corr_ms;     /* the S_1^T correlation, the dominant kernel */
     double starlet_ms;  /* starlet analysis with the per-coefficient sums */
     double final_ms;    /* the final reductions */
-    int launches;       /* kernels the call launched */
+    int launches;       /* kernels of the pass that the results come from, set-up included */
     int batch;          /* realisations per batch */
 } sr_noise_timing;
 

@@ -17,7 +17,9 @@
 // Work per batch of B realisations (all resident in L2):
 //   noise_draw_kernel      x[b]  = z / sigma_eff^                     (one Philox block a thread)
 //   noise_corr_kernel      y[b]  = S_1^T x[b]                          (FP32, 2 F^2 K^2 flop each), or
-//   noise_fft_kernel       the same by transforms (noise_fft.cu), where that is cheaper
+//   noise_fft_kernel       the same by transforms (noise_fft.cu), where that is cheaper and as accurate
+//                          (noise_level, in the first batch's draw, tells; if not, the call starts over
+//                          with the direct form)
 //   noise_row_kernel       t[b]  = row pass of level j on c_j[b]
 //   noise_col_stats_kernel c_{j+1}[b] = column pass; w = c_j - c_{j+1}; sum and sum of squares of
 //                          w over the batch, in a fixed order, into per-segment FP64 accumulators
@@ -62,16 +64,17 @@ __device__ __forceinline__ float uniform24(uint64_t w) { return (float)((w >> 40
 // starts at pixel 0 of its first realisation, so the pixel of number n0 + i is i mod F^2, in 32 bits
 // (Int) unless one realisation alone is larger than that: a 64-bit remainder per number cost as much
 // as the generator (5000 realisations at F = 128: 0.53 ms before, 0.43 ms with this).
+// Block b of nb.
 template <typename Int>
-__global__ void __launch_bounds__(256) noise_draw_kernel(const float *__restrict__ isig, int F, uint64_t seed,
-                                                         long long r0, int B, float *__restrict__ x) {
+__device__ __forceinline__ void noise_draw(const float *__restrict__ isig, int F, uint64_t seed, long long r0, int B,
+                                           float *__restrict__ x, int b, int nb) {
     const Int FF = (Int)F * F;
     const long long n0 = r0 * FF;
     const Int total = B * FF;
     const int lead = (int)(n0 & 3);  // the first block's numbers before the batch
     const long long blk0 = n0 >> 2;
     const Int nblk = (lead + total + 3) >> 2;
-    for (Int k = blockIdx.x * blockDim.x + threadIdx.x; k < nblk; k += gridDim.x * blockDim.x) {
+    for (Int k = b * (int)blockDim.x + (int)threadIdx.x; k < nblk; k += nb * (int)blockDim.x) {
         uint64_t c0 = (uint64_t)(blk0 + k), c1 = 0, c2 = 0, c3 = 0;
         philox4x64_10(c0, c1, c2, c3, seed, 0);
         float z[4];
@@ -218,7 +221,8 @@ __device__ __forceinline__ int reflect(int t, int F) { return t < 0 ? -t : (t > 
 
 // t[b][y][x] = sum_m h[m] c[b][y][reflect(x + m step)]
 __global__ void __launch_bounds__(256) noise_row_kernel(const float *__restrict__ c, float *__restrict__ t, int F,
-                                                        int step, long long total) {
+                                                        int step, long long total, const int *__restrict__ skip) {
+    if (skip && *skip) return;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         const int xx = (int)(idx % F);
@@ -374,6 +378,7 @@ __device__ __forceinline__ double inv_square(float sg) {
 //   are in flight together; one thread per fine pixel walking every epoch took 0.25 ms at E = 300,
 //   N = 64.
 // blocks n_isig + kx, kx < spec.L: column kx of the transform form's kernel spectrum (noise_spectrum).
+// block n_isig + spec.L, with spec.L > 0: the PSF's norm and peak (noise_peak).
 constexpr int kIsigWarps = 8;
 
 __device__ void noise_isig(const float *__restrict__ sigma, const float *__restrict__ s1, int N, int f, int E, int K,
@@ -453,14 +458,148 @@ __device__ void noise_spectrum(const float *__restrict__ s, int K, int kx, const
     }
 }
 
+// Norm^2 and position of the largest |s| (the first of equals), by one block.
+struct NoisePeak {
+    double norm2;
+    int qy, qx;
+};
+__device__ void noise_peak(const float *__restrict__ s, int K, NoisePeak *peak, double2 *red) {
+    double n2 = 0.0, top = -1.0;
+    int at = 0;
+    for (int q = threadIdx.x; q < K * K; q += blockDim.x) {
+        const double v = (double)__ldg(s + q);
+        n2 += v * v;
+        if (fabs(v) > top) {
+            top = fabs(v);
+            at = q;
+        }
+    }
+    __shared__ int s_at[kSpecMax];
+    red[threadIdx.x] = make_double2(n2, top);
+    s_at[threadIdx.x] = at;
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) {
+            const double2 a = red[threadIdx.x], b = red[threadIdx.x + w];
+            const int ia = s_at[threadIdx.x], ib = s_at[threadIdx.x + w];
+            const bool other = b.y > a.y || (b.y == a.y && ib < ia);
+            red[threadIdx.x] = make_double2(a.x + b.x, other ? b.y : a.y);
+            s_at[threadIdx.x] = other ? ib : ia;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *peak = NoisePeak{red[0].x, s_at[0] / K, s_at[0] % K};
+}
+
 __global__ void __launch_bounds__(32 * kIsigWarps)
 noise_setup_kernel(const float *__restrict__ sigma, const float *__restrict__ s1, int N, int f, int E, int K,
-                   int n_isig, float *__restrict__ isig, int *__restrict__ flag, NoiseSpec spec) {
+                   int n_isig, float *__restrict__ isig, int *__restrict__ flag, NoiseSpec spec, NoisePeak *peak) {
     __shared__ double2 w[kSpecMax], R[kSpecMax];
     if ((int)blockIdx.x < n_isig)
         noise_isig(sigma, s1, N, f, E, K, n_isig, isig, flag, reinterpret_cast<double (*)[32]>(w));
-    else
+    else if ((int)blockIdx.x < n_isig + spec.L)
         noise_spectrum(s1, K, blockIdx.x - n_isig, spec, w, R);
+    else
+        noise_peak(s1, K, peak, w);
+}
+
+// Whether the transforms are accurate enough for these inputs: *direct = 0, else 1 and the call takes the
+// direct correlation.  The rounding of a transform spreads over its whole image,
+// about 2^-24 of the image's rms level, while the direct sums round relative to what a pixel's own
+// window holds: where sigma_eff differs much over the grid, or a region is masked, a faint pixel
+// would lose accuracy (sigma rising by 1e6 across the grid: 0.1 % rms; a masked corner: noise of 1e-7 of
+// the level where there is none).  So the faintest pixel's level is compared with the rms: level^2 =
+// sum_q s[q]^2 isig[v + q - o]^2, the variance of y[v], over the taps within kLevelBox of the peak.
+// The direct sums round the more the longer they are.  Measured on the faintest pixels of a grid whose
+// halves differ in sigma (F = 128, first plane; rms / faintest level: direct / transforms, 1e-7): K = 15,
+// 1.8: 1.0 / 0.8, 2.8: 1.0 / 0.9, 5.2: 1.0 / 1.3; K = 21, 4.0: 2.3 / 2.0, 5.2: 2.2 / 2.2; K = 33, 5.2: 3.6 / 2.1, 10:
+// 3.6 / 4.2; K = 64, 9.2: 2.6 / 1.4 (the second plane equal there), 18: 2.5 / 2.7.  Hence K / 8, at least
+// 2.5: an even grid has 1.8 (a quarter of the PSF at its corners), a 300-epoch quasar field 3.2.
+constexpr int kLevelBox = 6, kLevelBlocks = 128;
+constexpr float kLevelRange = 1e12f;  // 1 / sigma_eff and the PSF's norm within 1e-12 .. 1e12: no overflow
+struct LevelPart {
+    float least, most;  // level^2, isig
+    double power;       // sum of isig^2
+};
+// Block b of nb.
+__device__ __noinline__ void noise_level(const float *__restrict__ isig, const float *__restrict__ s1, int F, int K, int L,
+                                         const NoisePeak *__restrict__ peak, LevelPart *part, int *done,
+                                         int *__restrict__ direct, int b, int nb) {
+    __shared__ LevelPart s_part[8];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = K / 2;
+    const int cy = peak->qy - kLevelBox, cx = peak->qx - kLevelBox;
+    LevelPart p{INFINITY, 0.f, 0.0};
+    for (int u = b * 256 + threadIdx.x; u < F * F; u += nb * 256) {
+        const int y = u / F, x = u - y * F;
+        float lv = 0.f;
+#pragma unroll 2
+        for (int a = 0; a <= 2 * kLevelBox; ++a) {
+            const int qy = cy + a, gy = y + qy - o;
+            if (qy < 0 || qy >= K || gy < 0 || gy >= F) continue;
+            float v[2 * kLevelBox + 1];
+#pragma unroll
+            for (int c = 0; c <= 2 * kLevelBox; ++c) {  // a row's loads together
+                const int qx = cx + c, gx = x + qx - o;
+                const bool in = qx >= 0 && qx < K && gx >= 0 && gx < F;
+                v[c] = in ? __ldg(s1 + qy * K + qx) * __ldg(isig + gy * F + gx) : 0.f;
+            }
+#pragma unroll
+            for (int c = 0; c <= 2 * kLevelBox; ++c) lv = fmaf(v[c], v[c], lv);
+        }
+        const float i = isig[u];
+        p.least = fminf(p.least, lv);
+        p.most = fmaxf(p.most, i);
+        p.power += (double)i * (double)i;
+    }
+    auto join = [](LevelPart a, LevelPart b) { return LevelPart{fminf(a.least, b.least), fmaxf(a.most, b.most), a.power + b.power}; };
+    auto warp_join = [&](LevelPart a) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1)
+            a = join(a, LevelPart{__shfl_down_sync(0xffffffffu, a.least, d), __shfl_down_sync(0xffffffffu, a.most, d),
+                                  __shfl_down_sync(0xffffffffu, a.power, d)});
+        return a;
+    };
+    p = warp_join(p);
+    if (lane == 0) s_part[warp] = p;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) p = join(p, s_part[k]);
+        part[b] = p;
+        __threadfence();
+        s_last = atomicAdd(done, 1) == nb - 1;
+    }
+    __syncthreads();
+    if (!s_last || warp != 0) return;
+    __threadfence();
+    LevelPart t{INFINITY, 0.f, 0.0};
+    for (int k = lane; k < nb; k += 32) t = join(t, part[k]);
+    t = warp_join(t);
+    if (lane == 0) {
+        const float norm = (float)sqrt(peak->norm2);
+        // the rms over a transform's L x L points; of one tile of several, at most the brightest pixel's
+        const float rms = norm * fminf(t.most, (float)sqrt(t.power / ((double)L * (double)L)));
+        const float limit = fmaxf(2.5f, (float)K / 8.f);
+        const bool even = sqrtf(t.least) * limit >= rms;  // false for a NaN
+        const bool range = t.most <= kLevelRange && t.most >= 1.f / kLevelRange && norm <= kLevelRange && norm >= 1.f / kLevelRange;
+        *direct = even && range ? 0 : 1;
+    }
+}
+
+template <typename Int>
+__global__ void __launch_bounds__(256) noise_draw_kernel(const float *__restrict__ isig, int F, uint64_t seed,
+                                                         long long r0, int B, float *__restrict__ x) {
+    noise_draw<Int>(isig, F, seed, r0, B, x, blockIdx.x, gridDim.x);
+}
+
+// The first batch's draw where the transforms may run: blocks [0, n_level) look at the level, beside it.
+template <typename Int>
+__global__ void __launch_bounds__(256)
+noise_first_draw_kernel(const float *__restrict__ isig, int F, uint64_t seed, int B, float *__restrict__ x, int n_level,
+                        const float *__restrict__ s1, int K, int L, const NoisePeak *__restrict__ peak, LevelPart *part,
+                        int *done, int *__restrict__ direct) {
+    if ((int)blockIdx.x < n_level) noise_level(isig, s1, F, K, L, peak, part, done, direct, blockIdx.x, n_level);
+    else noise_draw<Int>(isig, F, seed, 0, B, x, blockIdx.x - n_level, gridDim.x - n_level);
 }
 
 // Whether S_1^T runs as transforms (noise_fft.cu) rather than as the direct correlation, by cost per
@@ -587,10 +726,12 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
     float *isig, *xbuf, *cbuf, *wsc;
     double2 *scale_part;
     double *acc1, *acc2;
-    int *flag;
+    int *flag;  // flag, direct; J1 + 1 finishing counters
+    NoisePeak *peak = nullptr;
+    LevelPart *level_part = nullptr;
     ws.reserve(&acc1, (size_t)S * J1 * FF);
     ws.reserve(&acc2, (size_t)S * J1 * FF);
-    ws.reserve(&flag, 1 + J1);
+    ws.reserve(&flag, 3 + J1);
     const size_t zeroed = ws.bytes;
     ws.reserve(&isig, FF);
     ws.reserve(&xbuf, B * FF);
@@ -600,6 +741,8 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
     if (use_fft) {
         ws.reserve(&spec.S, (size_t)fft.L * fft.L);
         ws.reserve(&spec.tw, fft.L);
+        ws.reserve(&peak, 1);
+        ws.reserve(&level_part, kLevelBlocks);
         spec.L = fft.L;
         spec.R1 = fft.R1;
         spec.sh = fft.n == 1 ? K / 2 : 0;
@@ -629,71 +772,114 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
     };
 
     const int n_isig = (int)std::min<long long>(((long long)N * N + 31) / 32, sms * 8LL);
-    noise_setup_kernel<<<n_isig + spec.L, 32 * kIsigWarps, 0, st>>>(sigma_dev, s1_dev, N, f, E, K, n_isig, isig, flag,
-                                                                    spec);
+    noise_setup_kernel<<<n_isig + spec.L + (use_fft ? 1 : 0), 32 * kIsigWarps, 0, st>>>(sigma_dev, s1_dev, N, f, E, K,
+                                                                                        n_isig, isig, flag, spec, peak);
     ++launches;
-    for (long long r0 = 0; r0 < n_real; r0 += B) {
-        const int Bb = (int)std::min(B, (long long)n_real - r0);
+    const int n_level = (int)std::min<long long>((FF + 255) / 256, kLevelBlocks);
+    // The transforms' first batch runs before the host knows whether they are to be used: asking first would
+    // leave the GPU idle for the answer (a call of 400 us took 445).
+    bool fft_now = use_fft;
+    int found[2] = {0, 0};  // bad inputs; use the direct form
+    auto read_found = [&]() -> cudaError_t {
+        cudaError_t e = cudaMemcpyAsync(found, flag, sizeof found, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        return e;
+    };
+    auto start_over = [&]() -> cudaError_t {  // what the transforms' batches left
+        fft_now = false;
+        launches = 1;
+        return cudaMemsetAsync(ws.base, 0, zeroed, st);
+    };
+    cudaError_t e = cudaSuccess;
+    for (;;) {
+        for (long long r0 = 0; r0 < n_real; r0 += B) {
+            if (fft_now && r0 == B) {
+                e = read_found();
+                if (e == cudaSuccess && found[1]) {
+                    e = start_over();
+                    r0 = 0;
+                }
+                if (e != cudaSuccess) break;
+            }
+            const int Bb = (int)std::min(B, (long long)n_real - r0);
+            const int *skip = fft_now ? flag + 1 : nullptr;
+            if (timed) cudaEventRecord(ev[0], st);
+            const long long nblk = ((r0 + Bb) * FF - 1) / 4 - (r0 * FF) / 4 + 1;
+            const int gd = (int)std::min<long long>((nblk + 255) / 256, sms * 16LL);
+            const bool small = Bb * FF < (1LL << 30);
+            if (fft_now && r0 == 0) {
+                int *done = flag + 2 + J1;
+                if (small)
+                    noise_first_draw_kernel<int><<<n_level + gd, 256, 0, st>>>(isig, F, seed, Bb, xbuf, n_level, s1_dev, K,
+                                                                               spec.L, peak, level_part, done, flag + 1);
+                else
+                    noise_first_draw_kernel<long long><<<n_level + gd, 256, 0, st>>>(isig, F, seed, Bb, xbuf, n_level, s1_dev,
+                                                                                     K, spec.L, peak, level_part, done, flag + 1);
+            } else if (small) {
+                noise_draw_kernel<int><<<gd, 256, 0, st>>>(isig, F, seed, r0, Bb, xbuf);
+            } else {
+                noise_draw_kernel<long long><<<gd, 256, 0, st>>>(isig, F, seed, r0, Bb, xbuf);
+            }
+            if (timed) cudaEventRecord(ev[1], st);
+            if (fft_now) {
+                if ((rc = launch_noise_fft(fft, xbuf, spec.S, spec.tw, F, K, Bb, sms, skip, cbuf, st)) != SR_OK) {
+                    destroy_events();
+                    return rc;
+                }
+            } else {
+                noise_corr_kernel<<<dim3(tiles_x, tiles_y, Bb), kCorrThreads, corr_smem, st>>>(xbuf, s1_dev, F, K, KP, KC,
+                                                                                               cbuf);
+            }
+            if (timed) cudaEventRecord(ev[2], st);
+            const long long total = Bb * FF;
+            const int Sb = std::min(S, Bb);
+            for (int j = 0; j < J1; ++j) {
+                noise_row_kernel<<<(int)std::min<long long>((total + 255) / 256, sms * 16LL), 256, 0, st>>>(
+                    cbuf, xbuf, F, 1 << j, total, skip);
+                noise_col_stats_kernel<<<dim3((unsigned)((FF + 255) / 256), Sb), 256, 0, st>>>(
+                    cbuf, xbuf, F, 1 << j, Bb, Sb, J1, j, acc1, acc2);
+            }
+            launches += 2 + 2 * J1;
+            if (timed) {
+                cudaEventRecord(ev[3], st);
+                if ((e = cudaEventSynchronize(ev[3])) != cudaSuccess) break;
+                t_draw += elapsed(0, 1);
+                t_corr += elapsed(1, 2);
+                t_star += elapsed(2, 3);
+            }
+        }
+        if (e != cudaSuccess) {
+            destroy_events();
+            return cuda_fail(e, "noise propagation batch");
+        }
         if (timed) cudaEventRecord(ev[0], st);
-        const long long nblk = ((r0 + Bb) * FF - 1) / 4 - (r0 * FF) / 4 + 1;
-        const int gd = (int)std::min<long long>((nblk + 255) / 256, sms * 16LL);
-        if (Bb * FF < (1LL << 30)) noise_draw_kernel<int><<<gd, 256, 0, st>>>(isig, F, seed, r0, Bb, xbuf);
-        else noise_draw_kernel<long long><<<gd, 256, 0, st>>>(isig, F, seed, r0, Bb, xbuf);
-        if (timed) cudaEventRecord(ev[1], st);
-        if (use_fft) {
-            if ((rc = launch_noise_fft(fft, xbuf, spec.S, spec.tw, F, K, Bb, sms, cbuf, st)) != SR_OK) {
-                destroy_events();
-                return rc;
-            }
-        } else {
-            noise_corr_kernel<<<dim3(tiles_x, tiles_y, Bb), kCorrThreads, corr_smem, st>>>(xbuf, s1_dev, F, K, KP, KC,
-                                                                                           cbuf);
+        if (W_map_dev) {
+            const long long per = (long long)J1 * FF;
+            noise_map_kernel<<<(unsigned)((per + 255) / 256), 256, 0, st>>>(acc1, acc2, per, S, n_real, W_map_dev);
+            ++launches;
         }
-        if (timed) cudaEventRecord(ev[2], st);
-        const long long total = Bb * FF;
-        const int Sb = std::min(S, Bb);
-        for (int j = 0; j < J1; ++j) {
-            noise_row_kernel<<<(int)std::min<long long>((total + 255) / 256, sms * 16LL), 256, 0, st>>>(
-                cbuf, xbuf, F, 1 << j, total);
-            noise_col_stats_kernel<<<dim3((unsigned)((FF + 255) / 256), Sb), 256, 0, st>>>(
-                cbuf, xbuf, F, 1 << j, Bb, Sb, J1, j, acc1, acc2);
-        }
-        launches += 2 + 2 * J1;
-        if (timed) {
-            cudaEventRecord(ev[3], st);
-            const cudaError_t e = cudaEventSynchronize(ev[3]);
-            if (e != cudaSuccess) {
-                destroy_events();
-                return cuda_fail(e, "noise propagation batch");
-            }
-            t_draw += elapsed(0, 1);
-            t_corr += elapsed(1, 2);
-            t_star += elapsed(2, 3);
-        }
-    }
-    if (timed) cudaEventRecord(ev[0], st);
-    if (W_map_dev) {
-        const long long per = (long long)J1 * FF;
-        noise_map_kernel<<<(unsigned)((per + 255) / 256), 256, 0, st>>>(acc1, acc2, per, S, n_real, W_map_dev);
+        noise_scale_kernel<<<dim3(kScaleBlocks, J1), kScaleThreads, 0, st>>>(acc1, acc2, FF, J1, S, n_real, scale_part,
+                                                                               flag + 2, wsc);
         ++launches;
+        if (timed) cudaEventRecord(ev[4], st);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) {
+            destroy_events();
+            return cuda_fail(e, "noise propagation kernels");
+        }
+        if (W_host) e = cudaMemcpyAsync(W_host, wsc, sizeof(float) * J1, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = fft_now || !use_fft ? read_found() : cudaStreamSynchronize(st);
+        if (e == cudaSuccess && fft_now && found[1]) {  // one batch in all
+            e = start_over();
+            if (e == cudaSuccess) continue;
+        }
+        if (e != cudaSuccess) {
+            destroy_events();
+            return cuda_fail(e, "sr_noise_weights");
+        }
+        break;
     }
-    noise_scale_kernel<<<dim3(kScaleBlocks, J1), kScaleThreads, 0, st>>>(acc1, acc2, FF, J1, S, n_real, scale_part,
-                                                                           flag + 1, wsc);
-    ++launches;
-    if (timed) cudaEventRecord(ev[4], st);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        destroy_events();
-        return cuda_fail(e, "noise propagation kernels");
-    }
-    int hflag = 0;
-    e = cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && W_host) e = cudaMemcpyAsync(W_host, wsc, sizeof(float) * J1, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-        destroy_events();
-        return cuda_fail(e, "sr_noise_weights");
-    }
+    const int hflag = found[0];
     if (timed) {
         t_fin = elapsed(0, 4);
         timing->draw_ms = t_draw;

@@ -24,8 +24,8 @@ void noise_fft_gain(const NoiseFft &plan, double *gain);
 bool noise_fft_plan(int F, int K, int smem_optin, NoiseFft *plan);
 // Configures the transform kernel on the current device; *resident = its blocks per SM.
 sr_status noise_fft_prepare(const NoiseFft &plan, int *resident);
-// y[b] = S_1^T x[b] for the B realisations of a batch.
+// y[b] = S_1^T x[b] for the B realisations of a batch; nothing where *skip (on the device) is set.
 sr_status launch_noise_fft(const NoiseFft &plan, const float *x, const float2 *S, const float2 *tw, int F, int K, int B,
-                           int n_sms, float *y, cudaStream_t st);
+                           int n_sms, const int *skip, float *y, cudaStream_t st);
 
 }  // namespace sr

@@ -45,7 +45,8 @@ constexpr int nf_smem() {
 template <int L>
 __global__ void __launch_bounds__(kNfThreads, 1)
 noise_fft_kernel(const float *__restrict__ x, const float2 *__restrict__ S, const float2 *__restrict__ tw, int F, int K,
-                 int n, int T, int B, int n_items, float *__restrict__ y) {
+                 int n, int T, int B, int n_items, const int *__restrict__ skip, float *__restrict__ y) {
+    if (*skip) return;
     using G = Pr<L>;
     constexpr int R1 = G::R1, R2 = G::R2, P = G::P;
     float2 *Z = pr_dyn, *TWL = Z + G::ZN;
@@ -301,7 +302,7 @@ sr_status noise_fft_prepare(const NoiseFft &plan, int *resident) {
 }
 
 sr_status launch_noise_fft(const NoiseFft &plan, const float *x, const float2 *S, const float2 *tw, int F, int K, int B,
-                           int n_sms, float *y, cudaStream_t st) {
+                           int n_sms, const int *skip, float *y, cudaStream_t st) {
     const int items = (B + 1) / 2 * plan.n * plan.n;
     int threads = 0, occ = 0;
     switch (plan.L) {
@@ -310,7 +311,8 @@ sr_status launch_noise_fft(const NoiseFft &plan, const float *x, const float2 *S
         const sr_status rc = nf_block(noise_fft_kernel<LL>, nf_smem<LL>(), &threads, &occ);                    \
         if (rc != SR_OK) return rc;                                                                            \
         const int grid = items < occ * n_sms ? items : occ * n_sms;                                            \
-        noise_fft_kernel<LL><<<grid, threads, nf_smem<LL>(), st>>>(x, S, tw, F, K, plan.n, plan.T, B, items, y); \
+        noise_fft_kernel<LL><<<grid, threads, nf_smem<LL>(), st>>>(x, S, tw, F, K, plan.n, plan.T, B, items,   \
+                                                                   skip, y);                                   \
         break;                                                                                                 \
     }
         SR_NF_SIZES(SR_NF_RUN)
