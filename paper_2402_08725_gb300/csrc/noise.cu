@@ -361,16 +361,6 @@ __global__ void __launch_bounds__(kScaleThreads) noise_scale_kernel(const double
     }
 }
 
-// 1/sg^2 in FP64: an FP32 reciprocal and one Newton step (relative error below 1e-13; a division
-// is about three times the FP64 operations, which run at 2 a clock per SM), or the division itself
-// where sg^2 would leave the normal FP32 range.
-__device__ __forceinline__ double inv_square(float sg) {
-    const double s2 = (double)sg * (double)sg;
-    if (!(sg > 1e-15f && sg < 1e15f)) return 1.0 / s2;
-    const double r = (double)(1.f / (sg * sg));
-    return fma(r, fma(-s2, r, 1.0), r);
-}
-
 // The set-up of a call, one launch:
 // blocks [0, n_isig): 1/sigma_eff on the fine grid; flags (bit 0) a NaN or non-positive sigma and
 //   (bit 1) a non-finite PSF value.  A block takes 32 data pixels (lanes) and deals the epochs over
@@ -397,7 +387,7 @@ __device__ void noise_isig(const float *__restrict__ sigma, const float *__restr
             for (int i = warp; i < E; i += kIsigWarps) {
                 const float sg = __ldg(sigma + i * NN + p);
                 if (isnan(sg) || sg <= 0.f) bad = true;
-                else if (isfinite(sg)) iv += inv_square(sg);
+                else if (isfinite(sg)) iv += 1.0 / ((double)sg * (double)sg);
             }
         }
         if (bad) atomicOr(flag, 1);
