@@ -56,9 +56,9 @@ __device__ void split_store(const float2 *Z, float2 *out_a, float2 *out_b, int s
 }
 
 // The same for the two epochs of a kernel-spectra pair, side by side: out[ky][kx] = (re_a, re_b, im_a,
-// im_b); b zero without a second epoch.
+// im_b); b times back, zero without a second epoch.
 template <int L>
-__device__ void split_store_pair(const float2 *Z, float4 *out, bool hasb, int sh, const float2 *tw) {
+__device__ void split_store_pair(const float2 *Z, float4 *out, bool hasb, float back, int sh, const float2 *tw) {
     using G = Pr<L>;
     constexpr int H = G::H, HP = G::HP, P = G::P;
     const int rows = blockDim.x / HP;  // rows in parallel
@@ -79,7 +79,7 @@ __device__ void split_store_pair(const float2 *Z, float4 *out, bool hasb, int sh
             xa = cmul(make_float2(0.5f * (A.x + B.x), 0.5f * (A.y - B.y)), w);
             if (hasb) xb = cmul(make_float2(0.5f * (A.y + B.y), 0.5f * (B.x - A.x)), w);
         }
-        out[ky * HP + kx] = make_float4(xa.x, xb.x, xa.y, xb.y);
+        out[ky * HP + kx] = make_float4(xa.x, back * xb.x, xa.y, back * xb.y);
         wi += wstep;
         if (wi >= L) wi -= L;
     }
@@ -153,6 +153,21 @@ __device__ __noinline__ void cols_fwd_lead(float2 *Z, int ylim, const float2 *TW
 // placed instead at tau - tau_lo, so that the row passes touch only its Tk rows, and the shift is
 // restored on the spectrum (shift theorem):
 //   Khat[ky][kx] = W_L^((ky + kx) tau_lo) Khat'[ky][kx],   W_L = exp(-2 pi i / L).
+// The two epochs' PSFs need not be normalised alike, and a transform rounds relative to the larger of its
+// two images: the second epoch's kernel is brought to the first's magnitude by a power of two (exact) on
+// the way in and back on the way out, so that neither loses accuracy to the other.
+__shared__ unsigned s_top[2];  // bits of the largest |kappa| of either image; zero between items
+__device__ __forceinline__ void kappa_items_start() {
+    if (threadIdx.x < 2) s_top[threadIdx.x] = 0;
+    __syncthreads();
+}
+// the exponent that brings the second image's largest value to the first's (0 if either is zero,
+// subnormal or not finite)
+__device__ __forceinline__ int kappa_shift() {
+    const int a = (int)(s_top[0] >> 23), b = (int)(s_top[1] >> 23);
+    return a == 0 || b == 0 || a == 255 || b == 255 ? 0 : max(-100, min(100, a - b));
+}
+
 template <int L>
 __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__restrict__ kappa,
                                              float2 *__restrict__ khat, int item) {
@@ -165,11 +180,32 @@ __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__
     const int Tk = fd.Tk;
     const float *ka = kappa + ((long long)(2 * pr) * nph + ph) * Tk * Tk;
     const float *kb = 2 * pr + 1 < fd.E ? ka + (long long)nph * Tk * Tk : nullptr;
+    unsigned ta = 0, tb = 0;
     for (int t = threadIdx.x; t < Tk * Tk; t += blockDim.x) {
         const int y = t / Tk, x = t - y * Tk;
-        Z[y * P + pcol<L>(x)] = make_float2(ka[t], kb ? kb[t] : 0.f);
+        const float2 v = make_float2(ka[t], kb ? kb[t] : 0.f);
+        ta = max(ta, __float_as_uint(fabsf(v.x)));
+        tb = max(tb, __float_as_uint(fabsf(v.y)));
+        Z[y * P + pcol<L>(x)] = v;
+    }
+    if (kb) {
+        ta = __reduce_max_sync(0xffffffffu, ta);
+        tb = __reduce_max_sync(0xffffffffu, tb);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&s_top[0], ta);
+            atomicMax(&s_top[1], tb);
+        }
     }
     __syncthreads();
+    const int shift = kappa_shift();
+    if (shift != 0) {
+        const float by = ldexpf(1.f, shift);
+        for (int t = threadIdx.x; t < Tk * Tk; t += blockDim.x) {
+            const int y = t / Tk, x = t - y * Tk;
+            Z[y * P + pcol<L>(x)].y *= by;
+        }
+        __syncthreads();
+    }
     rows_fwd<L>(Z, 1, Tk, Tk, TWL);
     if constexpr (Pr<L>::R1 == 16) {
         if (4 * Tk <= L) cols_fwd_lead<L, 4>(Z, Tk, TWL);
@@ -180,13 +216,15 @@ __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__
     }
     const int sh = ((fd.tau_lo % L) + L) % L;  // tau_lo mod L
     float4 *out = reinterpret_cast<float4 *>(khat) + (long long)item * L * HP;
-    split_store_pair<L>(Z, out, kb != nullptr, sh, fd.fft_tw);
+    split_store_pair<L>(Z, out, kb != nullptr, ldexpf(1.f, -shift), sh, fd.fft_tw);
+    if (threadIdx.x < 2) s_top[threadIdx.x] = 0;
     __syncthreads();
 }
 
 __global__ void __launch_bounds__(kFftThreads, 1)
 fft_kappa_pair_kernel(FieldDev fd, const float *__restrict__ kappa, float2 *__restrict__ khat) {
     const int n_items = (fd.E + 1) / 2 * fd.f * fd.f;
+    kappa_items_start();
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         switch (fd.fft_L) {
 #define SR_PR_KCASE(LL)                                 \
@@ -205,6 +243,7 @@ fft_kappa_pair_kernel(FieldDev fd, const float *__restrict__ kappa, float2 *__re
 // phase); every block takes items in turn (the spectra live at each entry's fft_khat).
 __global__ void __launch_bounds__(kFftThreads, 1)
 fft_kappa_pair_batch_kernel(const FieldDev *__restrict__ fields, const int2 *__restrict__ items, int n_items) {
+    kappa_items_start();
     for (int j = blockIdx.x; j < n_items; j += gridDim.x) {
         const int2 it = items[j];
         const FieldDev &fd = fields[it.x];
