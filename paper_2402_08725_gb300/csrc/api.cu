@@ -2052,7 +2052,7 @@ static sr_status batch_io_prepare(sr_batch *b) {
         os[i + 1] = os[i] + (long long)e.E * e.K * e.K;
         ok[i + 1] = ok[i] + (long long)e.E * e.f * e.f * e.Tk * e.Tk;
         if (p->khat && !p->fft_big)
-            for (int j = 0; j < (e.E + 1) / 2 * e.f * e.f; ++j) items.push_back(make_int2(i, j));
+            for (int j = 0; j < fft_kappa_items(e.E, e.f); ++j) items.push_back(make_int2(i, j));
     }
     // items grouped by transform size: one launch per size with that size's block
     std::stable_sort(items.begin(), items.end(), [&](const int2 &a, const int2 &c) {

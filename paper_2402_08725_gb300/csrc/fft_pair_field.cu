@@ -55,10 +55,11 @@ __device__ void split_store(const float2 *Z, float2 *out_a, float2 *out_b, int s
     }
 }
 
-// The same for the two epochs of a kernel-spectra pair, side by side: out[ky][kx] = (re_a, re_b, im_a,
-// im_b); b times back, zero without a second epoch.
-template <int L>
-__device__ void split_store_pair(const float2 *Z, float4 *out, bool hasb, float back, int sh, const float2 *tw) {
+// The same for a transform of kernels, in the layout of an epoch pair, (re_a, re_b, im_a, im_b): both
+// epochs of one phase at out (b times back), or, ALONE, an epoch without a second, whose phases a and b go
+// to out and out_b (nullptr: there is no phase b) with zeros for the second epoch.
+template <int L, bool ALONE>
+__device__ void split_store_pair(const float2 *Z, float4 *out, float4 *out_b, float back, int sh, const float2 *tw) {
     using G = Pr<L>;
     constexpr int H = G::H, HP = G::HP, P = G::P;
     const int rows = blockDim.x / HP;  // rows in parallel
@@ -77,9 +78,14 @@ __device__ void split_store_pair(const float2 *Z, float4 *out, bool hasb, float 
             const float2 B = Z[krow<L>(neg_mod(ky, L)) * P + cxm];
             const float2 w = tw[wi];
             xa = cmul(make_float2(0.5f * (A.x + B.x), 0.5f * (A.y - B.y)), w);
-            if (hasb) xb = cmul(make_float2(0.5f * (A.y + B.y), 0.5f * (B.x - A.x)), w);
+            xb = cmul(make_float2(0.5f * (A.y + B.y), 0.5f * (B.x - A.x)), w);
         }
-        out[ky * HP + kx] = make_float4(xa.x, back * xb.x, xa.y, back * xb.y);
+        if (ALONE) {
+            out[ky * HP + kx] = make_float4(xa.x, 0.f, xa.y, 0.f);
+            if (out_b) out_b[ky * HP + kx] = make_float4(xb.x, 0.f, xb.y, 0.f);
+        } else {
+            out[ky * HP + kx] = make_float4(xa.x, back * xb.x, xa.y, back * xb.y);
+        }
         wi += wstep;
         if (wi >= L) wi -= L;
     }
@@ -148,7 +154,8 @@ __device__ __noinline__ void cols_fwd_lead(float2 *Z, int ylim, const float2 *TW
 }
 
 // Spectra of the folded PSF kernels (at set_psfs): item = epoch pair * f^2 + phase, the two epochs'
-// kernels of the phase as one complex image.  The phase kernel kappa_phi (Tk x Tk, taps tau_lo ..
+// kernels of the phase as one complex image; behind them, for an odd number of epochs, the last one's
+// phases two by two (fft_kappa_items).  The phase kernel kappa_phi (Tk x Tk, taps tau_lo ..
 // tau_lo + Tk - 1 on each axis, Tk <= L) belongs on the L x L circle with tap tau at tau mod L.  It is
 // placed instead at tau - tau_lo, so that the row passes touch only its Tk rows, and the shift is
 // restored on the spectrum (shift theorem):
@@ -168,44 +175,70 @@ __device__ __forceinline__ int kappa_shift() {
     return a == 0 || b == 0 || a == 255 || b == 255 ? 0 : max(-100, min(100, a - b));
 }
 
+// What an item holds: phases ph (and ph + 1 of a last single epoch) of epochs 2 pr and 2 pr + 1.
+struct KappaItem {
+    bool alone;
+    int pr, ph;
+};
+__device__ __forceinline__ KappaItem kappa_item(const FieldDev &fd, int item) {
+    const int nph = fd.f * fd.f, whole = fd.E / 2 * nph;  // items of two epochs
+    if (item >= whole) return {true, fd.E / 2, 2 * (item - whole)};
+    return {false, item / nph, item % nph};
+}
+
+// Not inlined, and with nothing kept for it across the passes: at 96 registers or less a 128-thread block of
+// the small sizes has one more neighbour on its SM than at 103 (100 fields of 20 epochs of 32 x 32 in 228 us).
+template <int L>
+__device__ __noinline__ void kappa_store(const FieldDev &fd, float2 *khat, int item) {
+    const KappaItem k = kappa_item(fd, item);
+    const int nph = fd.f * fd.f, sh = ((fd.tau_lo % L) + L) % L;  // tau_lo mod L
+    float4 *out = reinterpret_cast<float4 *>(khat) + ((long long)k.pr * nph + k.ph) * L * Pr<L>::HP;
+    if (k.alone)
+        split_store_pair<L, true>(pr_dyn, out, k.ph + 1 < nph ? out + L * Pr<L>::HP : nullptr, 1.f, sh, fd.fft_tw);
+    else
+        split_store_pair<L, false>(pr_dyn, out, nullptr, ldexpf(1.f, -kappa_shift()), sh, fd.fft_tw);
+}
+
 template <int L>
 __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__restrict__ kappa,
                                              float2 *__restrict__ khat, int item) {
     using G = Pr<L>;
-    constexpr int P = G::P, HP = G::HP;
+    constexpr int P = G::P;
     float2 *Z = pr_dyn, *TWL = Z + G::ZN;
     load_twl<L>(TWL, fd.fft_tw);
-    const int nph = fd.f * fd.f;
-    const int pr = item / nph, ph = item - pr * nph;
-    const int Tk = fd.Tk;
-    const float *ka = kappa + ((long long)(2 * pr) * nph + ph) * Tk * Tk;
-    const float *kb = 2 * pr + 1 < fd.E ? ka + (long long)nph * Tk * Tk : nullptr;
-    unsigned ta = 0, tb = 0;
-    for (int t = threadIdx.x; t < Tk * Tk; t += blockDim.x) {
-        const int y = t / Tk, x = t - y * Tk;
-        const float2 v = make_float2(ka[t], kb ? kb[t] : 0.f);
-        ta = max(ta, __float_as_uint(fabsf(v.x)));
-        tb = max(tb, __float_as_uint(fabsf(v.y)));
-        Z[y * P + pcol<L>(x)] = v;
-    }
-    if (kb) {
-        ta = __reduce_max_sync(0xffffffffu, ta);
-        tb = __reduce_max_sync(0xffffffffu, tb);
-        if ((threadIdx.x & 31) == 0) {
-            atomicMax(&s_top[0], ta);
-            atomicMax(&s_top[1], tb);
-        }
-    }
-    __syncthreads();
-    const int shift = kappa_shift();
-    if (shift != 0) {
-        const float by = ldexpf(1.f, shift);
+    {
+        const KappaItem k = kappa_item(fd, item);
+        const int nph = fd.f * fd.f, Tk = fd.Tk;
+        const float *ka = kappa + ((long long)(2 * k.pr) * nph + k.ph) * Tk * Tk;
+        const float *kb = !k.alone ? ka + (long long)nph * Tk * Tk : k.ph + 1 < nph ? ka + Tk * Tk : nullptr;
+        unsigned ta = 0, tb = 0;
         for (int t = threadIdx.x; t < Tk * Tk; t += blockDim.x) {
             const int y = t / Tk, x = t - y * Tk;
-            Z[y * P + pcol<L>(x)].y *= by;
+            const float2 v = make_float2(ka[t], kb ? kb[t] : 0.f);
+            ta = max(ta, __float_as_uint(fabsf(v.x)));
+            tb = max(tb, __float_as_uint(fabsf(v.y)));
+            Z[y * P + pcol<L>(x)] = v;
+        }
+        if (!k.alone) {
+            ta = __reduce_max_sync(0xffffffffu, ta);
+            tb = __reduce_max_sync(0xffffffffu, tb);
+            if ((threadIdx.x & 31) == 0) {
+                atomicMax(&s_top[0], ta);
+                atomicMax(&s_top[1], tb);
+            }
         }
         __syncthreads();
+        const int shift = kappa_shift();
+        if (shift != 0) {
+            const float by = ldexpf(1.f, shift);
+            for (int t = threadIdx.x; t < Tk * Tk; t += blockDim.x) {
+                const int y = t / Tk, x = t - y * Tk;
+                Z[y * P + pcol<L>(x)].y *= by;
+            }
+            __syncthreads();
+        }
     }
+    const int Tk = fd.Tk;
     rows_fwd<L>(Z, 1, Tk, Tk, TWL);
     if constexpr (Pr<L>::R1 == 16) {
         if (4 * Tk <= L) cols_fwd_lead<L, 4>(Z, Tk, TWL);
@@ -214,16 +247,15 @@ __device__ __noinline__ void kappa_item_pair(const FieldDev &fd, const float *__
     } else {
         cols_fwd<L>(Z, 1, Tk, TWL);
     }
-    const int sh = ((fd.tau_lo % L) + L) % L;  // tau_lo mod L
-    float4 *out = reinterpret_cast<float4 *>(khat) + (long long)item * L * HP;
-    split_store_pair<L>(Z, out, kb != nullptr, ldexpf(1.f, -shift), sh, fd.fft_tw);
+    kappa_store<L>(fd, khat, item);
+    __syncthreads();
     if (threadIdx.x < 2) s_top[threadIdx.x] = 0;
     __syncthreads();
 }
 
 __global__ void __launch_bounds__(kFftThreads, 1)
 fft_kappa_pair_kernel(FieldDev fd, const float *__restrict__ kappa, float2 *__restrict__ khat) {
-    const int n_items = (fd.E + 1) / 2 * fd.f * fd.f;
+    const int n_items = fft_kappa_items(fd.E, fd.f);
     kappa_items_start();
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         switch (fd.fft_L) {
@@ -239,8 +271,8 @@ fft_kappa_pair_kernel(FieldDev fd, const float *__restrict__ kappa, float2 *__re
     }
 }
 
-// The kernel spectra of many problems in one launch: items[j] = (table entry, epoch pair * f^2 +
-// phase); every block takes items in turn (the spectra live at each entry's fft_khat).
+// The kernel spectra of many problems in one launch: items[j] = (table entry, item of its problem);
+// every block takes items in turn (the spectra live at each entry's fft_khat).
 __global__ void __launch_bounds__(kFftThreads, 1)
 fft_kappa_pair_batch_kernel(const FieldDev *__restrict__ fields, const int2 *__restrict__ items, int n_items) {
     kappa_items_start();
@@ -528,7 +560,7 @@ sr_status launch_fft_kappa_pair_batch(const FieldDev *fields, const int2 *items,
 }
 
 void launch_fft_kappa_pair(const FieldDev &fd, const float *kappa, float2 *khat, cudaStream_t st) {
-    const int n_items = (fd.E + 1) / 2 * fd.f * fd.f;
+    const int n_items = fft_kappa_items(fd.E, fd.f);
     const int smem = fft_pair_field_smem(fd.fft_L);
     int threads = 0, occ = 0;
     kappa_block(fft_kappa_pair_kernel, smem, &threads, &occ);

@@ -54,7 +54,11 @@ sr_status configure_fft_pair_field(int optin, int *field_limit);  // called by c
 // spectra of a problem's folded kernels (set_psfs): [ceil(E/2)][f*f][L][L/2+2] of (re_a, re_b, im_a,
 // im_b) for epochs 2p and 2p + 1 (zero for a missing last one), the pad column zero
 void launch_fft_kappa_pair(const FieldDev &fd, const float *kappa, float2 *khat, cudaStream_t st);
-// the same for (entry, epoch pair * f^2 + phase) items of a table whose entries all have
+// Items (transforms) of that: one per phase of every two epochs, then one per two phases of a last single
+// epoch, as if it were two of half the phases: with a transform per phase 200 one-epoch fields of 64 x 64
+// took 58 us instead of 48.
+__host__ __device__ constexpr int fft_kappa_items(int E, int f) { return E / 2 * f * f + E % 2 * ((f * f + 1) / 2); }
+// the same for (entry, item) pairs of a table whose entries all have
 // transform size L (each entry's kappa and fft_khat), a persistent grid over n_sms SMs
 sr_status launch_fft_kappa_pair_batch(const FieldDev *fields, const int2 *items, int n_items, int L, int n_sms,
                                       cudaStream_t st);

@@ -38,3 +38,26 @@ def test_epochs_of_unlike_normalisation_keep_their_accuracy(N, f, K, scale, batc
     assert abs(loss - L_ref) <= 1e-6 * abs(L_ref)
     for name, epoch1 in (("a", slice(1, 2)), ("delta", slice(2, 4)), ("Gamma", slice(1, 2))):
         assert rel_l2(g[b[name]][epoch1], g_ref[b[name]][epoch1]) <= 1e-4, name
+
+
+@pytest.mark.parametrize("E", [1, 2, 5])
+@pytest.mark.parametrize("N,f,K", [(21, 2, 30), (27, 3, 33), (55, 1, 31)])  # four, nine and one phase
+@pytest.mark.parametrize("batched", [False, True])
+def test_odd_epochs_pair_their_phases(E, N, f, K, batched):
+    """The last epoch of an odd number: its phases share transforms two by two, an odd phase alone."""
+    import torch
+    from _helpers import check_deconv
+    from paper_2402_08725_gb300 import synthetic as syn
+    from paper_2402_08725_gb300.binding import Batch, Problem
+    fd = syn.small_deconv(seed=510 + N + E, E=E, N=N, f=f, K=K, M=2, J=3, lam=1.1)
+    prob = Problem.from_field(fd, conv_mode="fft")
+    P = torch.from_numpy(fd.params).cuda()
+    if batched:
+        batch = Batch([prob])
+        batch.set_psfs(torch.from_numpy(np.ascontiguousarray(fd.s, dtype=np.float32).reshape(-1)).cuda())
+        loss, grad = batch.loss_and_grad(P)
+        batch.close()
+    else:
+        loss, grad = prob.loss_and_grad(P)
+    prob.close()
+    check_deconv(fd, loss, grad.cpu().numpy())
