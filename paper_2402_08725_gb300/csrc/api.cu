@@ -452,18 +452,6 @@ static void fill_field_common(FieldDev &fd, sr_problem *p) {
     fd.Wmap = p->wmap_on ? p->wmap_dev : nullptr;
 }
 
-// Rows of the direct form's output tiles (64 columns wide): 64, or 32 or 16 for a field whose
-// (epoch, tile) items would not give every SM one.  A shorter tile stages more halo per output (Tk - 1
-// rows each) but runs more phases side by side in the block, so a field that leaves SMs idle gains
-// from it: 24 rotated epochs of 64 x 64 at Tk = 33, forward + adjoint kernel 357 us with 24 tiles of
-// 64 rows, 146 us with 96 of 16.  By the field's own shape, so that its sums do not depend on its
-// batch-mates.
-static int tile_rows(const sr_problem_desc &d, int n_sms) {
-    const long long across = (d.data_n + 63) / 64;
-    for (int rows : {64, 32})
-        if (d.n_epochs * across * ((d.data_n + rows - 1) / rows) >= n_sms) return rows;
-    return 16;
-}
 // Phase groups of a tile: the most phases at once that fit in the block's threads and in
 // shared memory (one group always).
 static int choose_pg(int nph, TileItem t, int Tk) {
@@ -622,6 +610,16 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
     chunk = std::max(2, std::min(kFftChunk, chunk)) & ~1;
     pl->chunk = chunk;
     pl->gp_cap = opt.gp_cap;
+    int rows = 64;  // of the direct form's tiles
+    if (pl->kind == SR_DECONV && !plain) {
+        std::vector<int> Es, Ns;
+        for (int i = 0; i < n; ++i)
+            if (probs[i]->desc.kind == SR_DECONV && !field_uses_fft(probs[i], opt)) {
+                Es.push_back(opt.epoch_limit > 0 ? std::min(probs[i]->desc.n_epochs, opt.epoch_limit) : probs[i]->desc.n_epochs);
+                Ns.push_back(probs[i]->desc.data_n);
+            }
+        rows = tile_rows(Es.data(), Ns.data(), (int)Es.size(), g_num_sms);
+    }
     for (int i = 0; i < n; ++i) {
         sr_problem *p = probs[i];
         if (p->desc.kind != pl->kind) return fail(SR_ERR_ARG, "a batch mixes problem kinds");
@@ -704,25 +702,27 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
             }
             const int nph = fd.f * fd.f;
             std::vector<TileItem> tiles;
-            const int rows = tile_rows(p->desc, g_num_sms);
+            const int across = (fd.N + 63) / 64;
             for (int y0 = 0; y0 < fd.N; y0 += rows)
                 for (int x0 = 0; x0 < fd.N; x0 += 64) {
                     TileItem t{};
                     t.field = i;
+                    t.slot = y0 / kTileBand * across + x0 / 64;  // of the epoch's
+                    t.band_stride = (short)across;
                     t.y0 = (short)y0;
                     t.x0 = (short)x0;
                     t.h = (short)std::min(rows, fd.N - y0);
                     t.w = (short)(((std::min(64, fd.N - x0)) + kR - 1) / kR * kR);
-                    t.pg = choose_pg(nph, t, fd.Tk);
+                    t.pg = (short)choose_pg(nph, t, fd.Tk);
                     tiles.push_back(t);
                 }
-            fd.n_tiles = (int)tiles.size();
+            fd.n_tiles = across * ((fd.N + kTileBand - 1) / kTileBand);  // partial sums per epoch
             fd.tile_slot = tslot;
             for (int e = 0; e < fd.E; ++e)
-                for (int k = 0; k < fd.n_tiles; ++k) {
-                    TileItem t = tiles[k];
+                for (const TileItem &tile : tiles) {
+                    TileItem t = tile;
                     t.epoch = e;
-                    t.slot = (int)(tslot + (long long)e * fd.n_tiles + k);
+                    t.slot += (int)(tslot + (long long)e * fd.n_tiles);
                     items.push_back(t);
                     smem_fwd = std::max(smem_fwd, tile_smem_bytes(t, fd.Tk, true));
                     smem_adj = std::max(smem_adj, tile_smem_bytes(t, fd.Tk, false));

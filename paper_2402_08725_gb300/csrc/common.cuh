@@ -102,13 +102,16 @@ __device__ __forceinline__ void shift_split(float s, int *n, float *t) {
 }
 
 // One output tile of one epoch: rows [y0, y0+h), cols [x0, x0+w) of the data
-// grid.  pg = number of thread groups working on different phases at once.
+// grid (h at most 64, y0 a multiple of kTileBand).  pg = number of thread groups working on different
+// phases at once.  Each band of kTileBand rows has its own partial sums, band b at slot + b band_stride; with
+// band_stride 0 their sum goes to slot.
+constexpr int kTileBand = 16;
 struct TileItem {
     int field;
     int epoch;
-    int slot;      // (epoch, tile) partial-sum slot
+    int slot;      // partial-sum slot of the first band
     short y0, x0, h, w;
-    int pg;
+    short pg, band_stride;
 };
 
 struct ChunkItem {

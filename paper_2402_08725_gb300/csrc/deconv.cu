@@ -175,9 +175,11 @@ fwd_kernel(const FieldDev *__restrict__ fields, const TileItem *__restrict__ ite
         __syncthreads();
         const int warp = tid >> 5, lane = tid & 31;
 
-        float acc[R];
+        // Each phase is summed on its own and the phases are added in order, however many run side by
+        // side: a pixel's bits do not depend on the tile it lies in.
+        float total[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = 0.f;
+        for (int r = 0; r < R; ++r) total[r] = 0.f;
 
         for (int iter = 0; iter < nph / G.PG; ++iter) {
             // stage F_phi = f_i[f m + phi] = h + point sources (zero outside the grid), one row per warp
@@ -247,28 +249,33 @@ fwd_kernel(const FieldDev *__restrict__ fields, const TileItem *__restrict__ ite
                 for (int jx = lane; jx < G.kpitch; jx += 32) dst[jx] = jx < Tk ? __ldg(srow - jx) : 0.f;
             }
             __syncthreads();
+            float acc[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = 0.f;
             if (G.g < G.PG)
                 corr_accumulate<R>(acc, smem + G.g * xsize + G.row * G.xpitch + G.chunk * R, G.xpitch,
                                    Kall + G.g * ksz, G.kpitch, Tk);
             __syncthreads();
-        }
-        // sum the phase groups (fixed order)
-        if (G.PG > 1) {
-            float *red = smem;
-            if (G.g >= 1 && G.g < G.PG) {
+            if (G.PG > 1) {
+                float *red = smem;
+                if (G.g >= 1 && G.g < G.PG) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) red[((G.g - 1) * G.h + G.row) * G.w + G.chunk * R + r] = acc[r];
+                    for (int r = 0; r < R; ++r) red[((G.g - 1) * G.h + G.row) * G.w + G.chunk * R + r] = acc[r];
+                }
+                __syncthreads();
             }
-            __syncthreads();
             if (G.g == 0) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) total[r] += acc[r];
                 for (int gg = 1; gg < G.PG; ++gg) {
 #pragma unroll
-                    for (int r = 0; r < R; ++r) acc[r] += red[((gg - 1) * G.h + G.row) * G.w + G.chunk * R + r];
+                    for (int r = 0; r < R; ++r) total[r] += smem[((gg - 1) * G.h + G.row) * G.w + G.chunk * R + r];
                 }
             }
+            if (G.PG > 1) __syncthreads();
         }
-        // residual, chi^2 and sum e (FP32 over the thread's R pixels, compensated across the
-        // block), e = -w r
+        // residual, chi^2 and sum e (FP32 over the thread's R pixels, compensated over each band of
+        // kTileBand rows), e = -w r
         float chi_r = 0.f, se_r = 0.f;
         const int py = t.y0 + G.row;
         if (G.g == 0 && py < N) {
@@ -278,7 +285,7 @@ fwd_kernel(const FieldDev *__restrict__ fields, const TileItem *__restrict__ ite
             for (int r = 0; r < R; ++r) {
                 const int px = t.x0 + G.chunk * R + r;
                 if (px < N) {
-                    const float Mv = acc[r] + bg;
+                    const float Mv = total[r] + bg;
                     const float res = __ldg(fd.d + base + px) - Mv;
                     const float wv = __ldg(fd.w + base + px);
                     chi_r += 0.5f * wv * res * res;
@@ -288,11 +295,41 @@ fwd_kernel(const FieldDev *__restrict__ fields, const TileItem *__restrict__ ite
                 }
             }
         }
-        double chi = 0.0, se = 0.0;
-        block_fsum2(FSum{chi_r, 0.f}, FSum{se_r, 0.f}, s_red, chi, se);
-        if (tid == 0) {
-            chi_part[t.slot] = chi;
-            se_part[t.slot] = se;
+        // one warp per band, its values in row order: the bits of a band's sums do not depend on the
+        // tile either (the staged tiles are free by now: h w / 8 floats of at least h w)
+        float2 *vals = reinterpret_cast<float2 *>(smem);
+        const int nch = G.w / R, bands = (G.h + kTileBand - 1) / kTileBand;
+        if (G.g == 0) vals[G.row * nch + G.chunk] = make_float2(chi_r, se_r);
+        __syncthreads();
+        if (warp < bands) {
+            const int n = min(kTileBand, G.h - warp * kTileBand) * nch;  // at most 64
+            const float2 *v = vals + warp * kTileBand * nch;
+            FSum c = fsum_zero(), s = fsum_zero();
+            for (int k = lane; k < n; k += 32) {
+                c = fsum_add(c, v[k].x);
+                s = fsum_add(s, v[k].y);
+            }
+            c = fsum_warp(c);
+            s = fsum_warp(s);
+            if (lane == 0) {
+                s_red[0][warp] = make_float2(c.hi, c.lo);
+                s_red[1][warp] = make_float2(s.hi, s.lo);
+            }
+        }
+        __syncthreads();
+        if (t.band_stride > 0) {
+            if (tid < bands) {
+                chi_part[t.slot + tid * t.band_stride] = fsum_value(FSum{s_red[0][tid].x, s_red[0][tid].y});
+                se_part[t.slot + tid * t.band_stride] = fsum_value(FSum{s_red[1][tid].x, s_red[1][tid].y});
+            }
+        } else if (tid == 0) {
+            FSum c = fsum_zero(), s = fsum_zero();
+            for (int k = 0; k < bands; ++k) {
+                c = fsum_add(c, FSum{s_red[0][k].x, s_red[0][k].y});
+                s = fsum_add(s, FSum{s_red[1][k].x, s_red[1][k].y});
+            }
+            chi_part[t.slot] = fsum_value(c);
+            se_part[t.slot] = fsum_value(s);
         }
         __syncthreads();
     }
@@ -739,11 +776,26 @@ int choose_tile_pg(int nph, TileItem t, int Tk, int smem_limit) {
     const int threads_per_group = t.h * (t.w / kR);
     for (int pg = 1; pg <= nph; ++pg) {
         if (nph % pg != 0 || pg * threads_per_group > kThreads) continue;
-        t.pg = pg;
+        t.pg = (short)pg;
         if (tile_smem_bytes(t, Tk, true) > smem_limit) continue;
         best = pg;
     }
     return best;
+}
+
+// A shorter tile stages more halo per output (Tk - 1 rows each) but runs more phases side by side in the block
+// and leaves fewer SMs idle, of which each takes two blocks: the tallest tile that gives two rounds of items
+// (64 rows) or one (32).  Rotated fields of 24 epochs of 64 x 64, us an evaluation with 64 / 32 / 16 rows: one
+// field (24 items of 64 rows) 407 / 268 / 203, four 463 / 426 / 409, eight 733 / 661 / 701, sixteen 1138 / 1167 /
+// 1233, 32 2125 / 2166 / 2389; of 10 epochs of 96 x 96, eight (320 items of 64) 890 / 691 / 722, sixteen 1186 /
+// 1197 / 1321.  The results do not depend on it.
+int tile_rows(const int *E, const int *N, int n, int n_sms) {
+    for (int rows : {64, 32}) {
+        long long items = 0;
+        for (int i = 0; i < n; ++i) items += (long long)E[i] * ((N[i] + 63) / 64) * ((N[i] + rows - 1) / rows);
+        if (items >= (rows == 64 ? 4LL : 2LL) * n_sms) return rows;
+    }
+    return 16;
 }
 
 sr_status configure_tile_kernels(int smem_fwd, int smem_adj) {

@@ -138,7 +138,7 @@ extern "C" sr_status sr_loss_and_grad_noalloc(const sr_problem_desc *desc, const
             t.x0 = (short)x0;
             t.h = (short)std::min(64, N - y0);
             t.w = (short)((std::min(64, N - x0) + kR - 1) / kR * kR);
-            t.pg = choose_tile_pg(nph, t, Tk, optin - kTileStaticReserve);
+            t.pg = (short)choose_tile_pg(nph, t, Tk, optin - kTileStaticReserve);
             tt.t[tt.n++] = t;
             smem_fwd = std::max(smem_fwd, tile_smem_bytes(t, Tk, true));
             smem_adj = std::max(smem_adj, tile_smem_bytes(t, Tk, false));

@@ -1,4 +1,5 @@
 """The host's rules that choose a kernel, a tile or a schedule, on the CPU."""
+import ctypes
 import subprocess
 
 from paper_2402_08725_gb300 import build
@@ -16,3 +17,23 @@ def test_an_epoch_without_a_second_pairs_its_phases(tmp_path):
     """Transforms of the kernel spectra: one per phase of two epochs, half as many for a single one."""
     calls = "".join(f'  printf("%d\\n", sr::fft_kappa_items({E}, {f}));\n' for E in (1, 2, 3, 8) for f in (1, 2, 3))
     assert _run_cpp(tmp_path, calls) == [1, 2, 5, 1, 4, 9, 2, 6, 14, 4, 16, 36]
+
+
+def _rule(name):
+    """A host function of the library that no C header declares."""
+    from paper_2402_08725_gb300 import _native
+    return getattr(ctypes.CDLL(_native.load()._name), name)
+
+
+def _ints(v):
+    return (ctypes.c_int * len(v))(*v)
+
+
+def test_tile_height_is_the_tables():
+    """A field that leaves SMs idle alone takes short tiles; the same field in a batch that fills them does not
+    pay their halo."""
+    rows = _rule("_ZN2sr9tile_rowsEPKiS1_ii")
+    for n, want in ((1, 16), (4, 16), (8, 32), (16, 32), (32, 64)):
+        assert rows(_ints([24] * n), _ints([64] * n), n, 152) == want
+    assert rows(_ints([300]), _ints([64]), 1, 152) == 32
+    assert rows(_ints([]), _ints([]), 0, 152) == 16
