@@ -12,9 +12,9 @@
 // and two T planes (J, J+1) used alternately; T_0 ends in plane J.
 //
 // Four ways to run, chosen per field (starlet_form) and table:
-//  * clusters (grids up to 256 pixels in tables too small to fill the GPU): all levels of a field in
-//    one launch, on a cluster of 8 blocks that take the comb bands below, with a cluster barrier
-//    between levels instead of a launch (see starlet_cluster_kernel).
+//  * clusters (grids up to 256 pixels in tables of a few fields): all levels of a field in one launch, on
+//    a cluster of 8 blocks that take the comb bands below, with a cluster barrier between levels instead
+//    of a launch (see starlet_cluster_kernel).
 //  * comb bands (most fields): the rows rho, rho + s, rho + 2 s, ... of level j (step s = 2^j)
 //    are one column tap apart, so a block taking 16 consecutive rows of one such comb stages
 //    only 20 input rows at any level; otherwise the same as the bands below, whose arithmetic
@@ -691,15 +691,23 @@ int starlet_forms_single(int F, int J, bool map) {
 
 int starlet_comb_rows_of(int forms) { return (forms & kStarletRows8) ? 8 : (forms & kStarletRows4) ? 4 : kCombRows; }
 
-// Rows per comb block for a table of comb-band fields (F, J of each): 16, or 8 or 4, and clusters, when
-// the table's level-0 blocks would not fill twice the SMs.  The results do not depend on it (the
-// prior's partial sums are kept per 4-row group).  Returns the forms bit to add (0 for 16 rows).
+// Rows per comb block for a table of comb-band fields (F, J of each): 16, or 8 or 4 when the table's
+// level-0 blocks would not fill twice the SMs; and clusters for those of at most kClusterMaxF when they take
+// at most two thirds of the SMs, so that all run at once beside the chi^2 kernels (a cluster's blocks must
+// be free together).  Fields of 20 epochs, us an evaluation in clusters / level by level: 64 x 64 grids, 8
+// fields 66 / 78, 16 95 / 82, 64 224 / 141; 128 x 128, 8 84 / 93, 12 104 / 111, 16 133 / 114, 32 212 / 164; 256 x
+// 256, 8 170 / 177, 12 209 / 204, 16 292 / 270.  The results do not depend on it (the prior's partial sums are
+// kept per 4-row group).  Returns the forms bits to add (0 for 16 rows, level by level).
 int starlet_comb_rows_bits(const int *F, const int *J, int n, int n_sms) {
-    long long blocks = 0;
+    long long blocks = 0, clusters = 0;
     for (int i = 0; i < n; ++i)
-        if (starlet_form(F[i], J[i]) == 3) blocks += comb_chunks(F[i], 1);
+        if (starlet_form(F[i], J[i]) == 3) {
+            blocks += comb_chunks(F[i], 1);
+            if (F[i] <= kClusterMaxF) ++clusters;
+        }
     if (blocks == 0 || blocks >= 2LL * n_sms) return 0;
-    return (2 * blocks >= 2LL * n_sms ? kStarletRows8 : kStarletRows4) | kStarletClusterBit;
+    const int rows = 2 * blocks >= 2LL * n_sms ? kStarletRows8 : kStarletRows4;
+    return rows | (clusters > 0 && 3 * clusters * kClusterBlocks <= 2LL * n_sms ? kStarletClusterBit : 0);
 }
 
 int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, const ChunkItem *chunks,
@@ -733,7 +741,7 @@ int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, co
     const bool map = (forms & kStarletMapBit) != 0;
     // comb-band fields: in clusters up to kClusterMaxF when the table asks for it, the others (if any)
     // level by level
-    const bool clusters = (forms & 8) != 0 && (forms & kStarletClusterBit) != 0 && (n_fields > 1 || Fmax <= kClusterMaxF);
+    const bool clusters = (forms & kStarletClusterBit) != 0;
     const int above = clusters ? kClusterMaxF : 0;
     const bool combs = (forms & 8) != 0 && Fmax > above;
     // comb bands: s combs of comb_chunks blocks at level j; staging of 2 (cr + 4) (forward) or

@@ -37,3 +37,14 @@ def test_tile_height_is_the_tables():
         assert rows(_ints([24] * n), _ints([64] * n), n, 152) == want
     assert rows(_ints([300]), _ints([64]), 1, 152) == 32
     assert rows(_ints([]), _ints([]), 0, 152) == 16
+
+
+def test_clusters_only_where_they_run_at_once():
+    """Starlet clusters: grids up to 256 pixels, in tables whose clusters leave a third of the SMs free."""
+    bits, cluster = _rule("_ZN2sr22starlet_comb_rows_bitsEPKiS1_ii"), 128
+
+    def has(*F):
+        return bool(bits(_ints(F), _ints([4] * len(F)), len(F), 152) & cluster)
+
+    assert has(64) and has(*[128] * 12) and has(256) and has(420, 128)
+    assert not has(*[64] * 16) and not has(*[256] * 16) and not has(420) and not has(600, 300)
