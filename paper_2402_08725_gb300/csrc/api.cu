@@ -948,24 +948,29 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
                                pl->l1_part, pl->losses, pl->total, st);
         return n;
     }
-    // The priors run beside the h spectra when they are one launch each (clusters), before the chunk
-    // kernel takes every SM (300 epochs of 64 x 64: 153 us an evaluation when launched after it);
-    // level by level they are launched after the chi^2 kernels, whose chain is the longer one.
+    // A prior with clusters (one launch for their fields) runs beside the h spectra, before the chunk kernel
+    // takes every SM (300 epochs of 64 x 64: 153 us an evaluation when launched after it; four fields of 200 x
+    // 200 with one of 420 x 420, which goes level by level, 285 against 290); one that is level by level alone
+    // is launched after the chi^2 kernels, whose chain is the longer one (700 x 700: 203 us, 223 before them).
     cudaStream_t prior = pl->prior.fork(st), pts = pl->n_sh > 0 ? pl->pts.fork(st) : st;
-    auto launch_priors = [&]() {
+    auto launch_prior = [&]() {
         n += launch_starlet(pl->d_fields, pl->n_fields, pl->Fmax, pl->starlet_forms, pl->d_chunks, pl->n_chunks,
                             pl->Jmax, params, pl->l1_part, prior);
         if (pl->l1_sum) {
             launch_l1_sum(pl->d_fields, pl->n_fields, pl->l1_part, pl->l1_sum, prior);
             ++n;
         }
+    };
+    auto launch_pts = [&]() {
         if (pl->n_sh > 0)
             n += launch_pts_prior(pl->d_sh, pl->d_fields, pl->n_sh, pl->sh_Fmax, pl->sh_Mmax, pl->sh_starlet_forms,
                                   pl->d_sh_chunks, pl->n_sh_chunks, pl->sh_Jmax, params, pl->abar, pl->pbar, pl->l1_pts,
                                   pl->pts_g, pts);
     };
     const bool early = (pl->starlet_forms & kStarletClusterBit) != 0;
-    if (early) launch_priors();
+    const bool pts_early = (pl->sh_starlet_forms & kStarletClusterBit) != 0;
+    if (early) launch_prior();
+    if (pts_early) launch_pts();
     cudaMemsetAsync(pl->d_counters, 0, 4 * sizeof(int), st);
     cudaEvent_t *ev = nullptr;
     if (pl->profiling && !pl->prof_ev.empty()) {
@@ -1011,7 +1016,8 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
     for (size_t b = 0; b < pl->big_fields.size(); ++b)
         n += launch_big_adj(pl->h_fields[pl->big_fields[b]], pl->big_buf[b], st);
     if (ev) cudaEventRecord(ev[3], st);
-    if (!early) launch_priors();
+    if (!early) launch_prior();
+    if (!pts_early) launch_pts();
     pl->prior.join(prior, st);
     if (pl->n_items > 0) {
         launch_hgrad(pl->d_fields, pl->d_chunks, pl->n_chunks, pl->gbuf, grad, params, st);
