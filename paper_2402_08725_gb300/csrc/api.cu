@@ -181,9 +181,9 @@ struct Branch {
         if (stream) cudaStreamDestroy(stream);
     }
     sr_status open() {
-        SR_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
-        SR_CUDA(cudaEventCreateWithFlags(&forked, cudaEventDisableTiming));
-        SR_CUDA(cudaEventCreateWithFlags(&joined, cudaEventDisableTiming));
+        if (!forked) SR_CUDA(cudaEventCreateWithFlags(&forked, cudaEventDisableTiming));
+        if (!joined) SR_CUDA(cudaEventCreateWithFlags(&joined, cudaEventDisableTiming));
+        if (!stream) SR_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
         return SR_OK;
     }
     // the branch's stream, ordered after everything queued on `st` so far; `st` itself when not open
@@ -254,6 +254,7 @@ struct Plan {
     // optimiser
     uint8_t *d_group = nullptr;
     float *opt_m = nullptr, *opt_v = nullptr, *grad_int = nullptr, *params_int = nullptr;
+    bool opt_ready = false;  // the optimiser's buffers are all there, the moments set
     long long *d_t = nullptr;
     float *d_bc = nullptr;
     double **d_hist_ptr = nullptr;
@@ -1139,15 +1140,16 @@ static sr_status ensure_plan(sr_problem *p) {
 }
 
 static sr_status ensure_opt_buffers(Plan *pl) {
-    if (pl->opt_m) return SR_OK;
+    if (pl->opt_ready) return SR_OK;
     sr_status st;
-    if ((st = pl->arena.alloc(&pl->opt_m, pl->n_params)) != SR_OK) return st;
-    if ((st = pl->arena.alloc(&pl->opt_v, pl->n_params)) != SR_OK) return st;
-    if ((st = pl->arena.alloc(&pl->grad_int, pl->n_params)) != SR_OK) return st;
+    // a call that runs out of memory on the way leaves what it has to the next one
+    for (float **p : {&pl->opt_m, &pl->opt_v, &pl->grad_int})
+        if (!*p && (st = pl->arena.alloc(p, pl->n_params)) != SR_OK) return st;
     if (!pl->plain && (st = pl->step.open()) != SR_OK) return st;
     SR_CUDA(cudaMemset(pl->opt_m, 0, sizeof(float) * pl->n_params));
     SR_CUDA(cudaMemset(pl->opt_v, 0, sizeof(float) * pl->n_params));
     SR_CUDA(cudaMemset(pl->d_t, 0, sizeof(long long)));
+    pl->opt_ready = true;
     return SR_OK;
 }
 
@@ -1527,7 +1529,7 @@ sr_status sr_set_lambda_pts(sr_problem *p, double lambda_pts) {
                 p->plan = old;
                 return st;
             }
-            if (old->opt_m) {  // the optimiser's state carries over
+            if (old->opt_ready) {  // the optimiser's state carries over
                 if ((st = ensure_opt_buffers(p->plan)) != SR_OK) return st;
                 Plan *pl = p->plan;
                 SR_CUDA(cudaMemcpyAsync(pl->opt_m, old->opt_m, sizeof(float) * pl->n_params, cudaMemcpyDeviceToDevice,
