@@ -238,7 +238,7 @@ struct Plan {
     std::vector<BigBuffers> big_buf;
     // fields whose channel moves with the epoch shifts: their shift gradients (2 per epoch)
     float *hs = nullptr;
-    int hs_Emax = 0;
+    int hs_Emax = 0, hs_Fmax = 0;
     // point-source prior (Eq. 11, third term): shadow entries of the fields that have it
     int n_sh = 0, sh_Fmax = 0, sh_Jmax = 0, sh_Mmax = 0, n_sh_chunks = 0;
     int sh_starlet_forms = 0;
@@ -700,6 +700,7 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
                 fd.hs_off = hs_len;
                 hs_len += 2LL * fd.E;
                 pl->hs_Emax = std::max(pl->hs_Emax, fd.E);
+                pl->hs_Fmax = std::max(pl->hs_Fmax, fd.F);
             }
             const int nph = fd.f * fd.f;
             std::vector<TileItem> tiles;
@@ -1011,7 +1012,7 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
         ++n;
     }
     if (pl->hs) {
-        launch_hshift_grad(pl->d_fields, pl->n_fields, pl->hs_Emax, params, pl->gbuf, pl->hs, src);
+        launch_hshift_grad(pl->d_fields, pl->n_fields, pl->hs_Emax, pl->hs_Fmax, params, pl->gbuf, pl->hs, src);
         ++n;
     }
     for (size_t b = 0; b < pl->big_fields.size(); ++b)

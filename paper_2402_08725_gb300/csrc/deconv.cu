@@ -556,8 +556,9 @@ hgrad_kernel(const FieldDev *__restrict__ fields, const ChunkItem *__restrict__ 
 // The moved channel's part of dL/d delta_i = f sum_u G_i(u) d(T h)(u)/d s, with d(T h)/d s_x =
 // -[(1 - t_y)(h(y0, x0 + 1) - h(y0, x0)) + t_y (h(y0 + 1, x0 + 1) - h(y0 + 1, x0))] (and the same with
 // the axes swapped), (x0, y0) = u + n.  Block (epoch, field); compensated FP32 sums in fixed order.
-// 1024 threads per block: with 256 a 24-epoch field's 24 blocks took 59 us, now 30 (64 pixels of gathers per
-// thread in a row).
+// About 16 pixels per thread (hshift_threads): 24 epochs of F = 128 take 30 us with 1024 threads a block and
+// 59 with 256, 64 fields of 8 epochs of F = 64 45 with 1024 and 27 with 256.  The count is the field's own, a
+// wider block's other threads idle, so that the sums' order does not depend on the table.
 constexpr int kShiftThreads = 1024;
 __global__ void __launch_bounds__(kShiftThreads)
 hshift_grad_kernel(const FieldDev *__restrict__ fields, const float *__restrict__ params,
@@ -578,7 +579,8 @@ hshift_grad_kernel(const FieldDev *__restrict__ fields, const float *__restrict_
     const float2 cs = fd.rot ? fd.rot[i] : make_float2(1.f, 0.f);
     const float2 sh = make_float2((float)f * cpar[2 * i], (float)f * cpar[2 * i + 1]);
     FSum sx = fsum_zero(), sy = fsum_zero();
-    for (int q = threadIdx.x; q < F * F; q += blockDim.x) {
+    const int nt = hshift_threads(F);
+    for (int q = (int)threadIdx.x < nt ? threadIdx.x : F * F; q < F * F; q += nt) {
         const int ph = q / (N * N), m = q - ph * N * N;
         const int uy = f * (m / N) + ph / f, ux = f * (m % N) + ph % f;
         const float G = Gi[q];
@@ -605,7 +607,7 @@ hshift_grad_kernel(const FieldDev *__restrict__ fields, const float *__restrict_
     __syncthreads();
     if (threadIdx.x == 0) {
         FSum ax = fsum_zero(), ay = fsum_zero();
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        for (int w = 0; w < nt / 32; ++w) {
             ax = fsum_add(ax, FSum{s_red[w].x, s_red[w].y});
             ay = fsum_add(ay, FSum{s_red[w].z, s_red[w].w});
         }
@@ -833,9 +835,9 @@ void launch_hgrad(const FieldDev *fields, const ChunkItem *chunks, int n_chunks,
     hgrad_kernel<<<n_chunks * kHgGroups, 256, 0, st>>>(fields, chunks, n_chunks, gbuf, grad, params);
 }
 
-void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, const float *params, const float *gbuf,
-                        float *hs, cudaStream_t st) {
-    hshift_grad_kernel<<<dim3(E_max, n_fields), kShiftThreads, 0, st>>>(fields, params, gbuf, hs);
+void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, int F_max, const float *params,
+                        const float *gbuf, float *hs, cudaStream_t st) {
+    hshift_grad_kernel<<<dim3(E_max, n_fields), hshift_threads(F_max), 0, st>>>(fields, params, gbuf, hs);
 }
 
 void launch_l1_sum(const FieldDev *fields, int n_fields, const double *l1_part, double *l1_sum, cudaStream_t st) {

@@ -28,9 +28,14 @@ void launch_psgrad(const FieldDev *fields, const int4 *ps_items, int n, const fl
                    float *ps_da, float *ps_du, cudaStream_t st);
 void launch_hgrad(const FieldDev *fields, const ChunkItem *chunks, int n_chunks, const float *gbuf, float *grad,
                   const float *params, cudaStream_t st);
-// the moved extended channel's part of dL/d delta_i (fields with translate set; grid E_max x fields)
-void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, const float *params, const float *gbuf,
-                        float *hs, cudaStream_t st);
+// threads of the shift gradient's block that take a field of F x F
+__host__ __device__ constexpr int hshift_threads(int F) {
+    return F * F / 16 < 128 ? 128 : F * F / 16 > 1024 ? 1024 : (F * F / 16 + 31) / 32 * 32;
+}
+// the moved extended channel's part of dL/d delta_i (fields with translate set, of at most E_max epochs and
+// F_max fine pixels; grid E_max x fields)
+void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, int F_max, const float *params,
+                        const float *gbuf, float *hs, cudaStream_t st);
 // pts_fields / l1_pts / pts_g: the point-source prior's table and outputs (launch_pts_prior), or
 // nullptr when no field of the table has the term
 // Returns its launches.

@@ -48,3 +48,9 @@ def test_clusters_only_where_they_run_at_once():
 
     assert has(64) and has(*[128] * 12) and has(256) and has(420, 128)
     assert not has(*[64] * 16) and not has(*[256] * 16) and not has(420) and not has(600, 300)
+
+
+def test_shift_gradient_threads_follow_the_grid(tmp_path):
+    """About 16 pixels a thread, whole warps, 128 to 1024 threads."""
+    got = _run_cpp(tmp_path, "".join(f'  printf("%d\\n", sr::hshift_threads({F}));\n' for F in (5, 64, 90, 128, 1536)))
+    assert got == [128, 256, 512, 1024, 1024]

@@ -60,3 +60,32 @@ def test_tile_heights_agree_and_match_oracle(E, N, f, K, M, frame):
         for p in probs:
             p.close()
     alone.close()
+
+
+def test_moved_fields_of_unlike_grids_equal_single_ones():
+    """The shift gradient's sums are each field's own, whatever the widest field of the table is."""
+    import torch
+    from paper_2402_08725_gb300 import synthetic as syn
+    from paper_2402_08725_gb300.binding import Batch, Problem
+    fields = [syn.small_deconv(seed=4500 + N, E=E, N=N, f=2, K=11, M=1, J=3, lam=1.0)
+              for E, N in ((3, 10), (2, 33), (4, 47), (1, 70))]
+
+    def problem(fd):
+        p = Problem.from_field(fd)
+        p.set_translate_h(True)
+        return p
+
+    probs = [problem(fd) for fd in fields]
+    batch = Batch(probs)
+    losses = torch.empty(len(fields), dtype=torch.float64, device="cuda")
+    _, g = batch.loss_and_grad(torch.from_numpy(batch.pack([fd.params for fd in fields])).cuda(), losses=losses)
+    for i, fd in enumerate(fields):
+        alone = problem(fd)
+        loss, grad = alone.loss_and_grad(torch.from_numpy(fd.params).cuda())
+        o = batch.offsets[i]
+        assert losses[i].item() == loss and torch.equal(g[o:o + fd.n_params], grad)
+        check_deconv(fd, loss, grad.cpu().numpy(), shifted=True)
+        alone.close()
+    batch.close()
+    for p in probs:
+        p.close()
