@@ -238,6 +238,7 @@ struct Plan {
     std::vector<BigBuffers> big_buf;
     // fields whose channel moves with the epoch shifts: their shift gradients (2 per epoch)
     float *hs = nullptr;
+    int n_direct_chunks = 0;  // of direct-form fields
     int hs_Emax = 0, hs_Fmax = 0;
     // point-source prior (Eq. 11, third term): shadow entries of the fields that have it
     int n_sh = 0, sh_Fmax = 0, sh_Jmax = 0, sh_Mmax = 0, n_sh_chunks = 0;
@@ -696,6 +697,7 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
             smem_fx = std::max(smem_fx, fft_pair_smem_bytes(L, fd.M, fd.f, G));
         } else if (pl->kind == SR_DECONV && !plain) {
             gbuf += (long long)fd.E * fd.f * fd.f * fd.N * fd.N;
+            pl->n_direct_chunks += fd.n_chunks;
             if (fd.translate) {
                 fd.hs_off = hs_len;
                 hs_len += 2LL * fd.E;
@@ -1022,7 +1024,7 @@ static int run_eval(Plan *pl, const float *params, float *grad, cudaStream_t st,
     if (!pts_early) launch_pts();
     pl->prior.join(prior, st);
     if (pl->n_items > 0) {
-        launch_hgrad(pl->d_fields, pl->d_chunks, pl->n_chunks, pl->gbuf, grad, params, st);
+        launch_hgrad(pl->d_fields, pl->d_chunks, pl->n_chunks, pl->n_direct_chunks, g_num_sms, pl->gbuf, grad, params, st);
         ++n;
     }
     if (pl->n_fft_items > 0) {

@@ -452,13 +452,11 @@ __global__ void psgrad_kernel(const FieldDev *__restrict__ fields, const int4 *_
     }
 }
 
-// dL/dh[u] = T0[u] + sum_i G_i[u] over the polyphase indexes q = phi*N*N + m.  A block takes a quarter
-// of a 256-pixel chunk: 64 pixels by kHgGroups groups of epochs (group g the epochs i = g mod 4 of
-// the whole quadruples, group 0 also the rest), whose sums are joined as (0 + 1) + (2 + 3).  A field
-// of few chunks is bound by the chain of each pixel's gathers over its epochs (rotated frames test 9
-// candidates per epoch): with one thread per pixel a 24-epoch field of 64 x 64 took 76 us on 64
-// blocks, with four 26 us on 256.
-constexpr int kHgGroups = 4, kHgPixels = 256 / kHgGroups;
+// dL/dh[u] = T0[u] + sum_i G_i[u] over the polyphase indexes q = phi*N*N + m, in four interleaved sums over
+// the epochs (i = g mod 4 of the whole quadruples, g = 0 also the rest), joined as (0 + 1) + (2 + 3).  SPLIT
+// = 4: a block takes a quarter of a 256-pixel chunk, 64 pixels by the four sums; SPLIT = 1: a chunk, each
+// thread all four sums of a pixel.  The same bits; which one by the table (launch_hgrad).
+constexpr int kHgGroups = 4;
 
 // the bilinear gather of one epoch's adjoint image at pixel (vx, vy)
 __device__ __forceinline__ float hgrad_rotated(const FieldDev &fd, const float *__restrict__ Gi, float2 cs, float2 sh,
@@ -511,23 +509,27 @@ __device__ __forceinline__ float hgrad_shifted(const FieldDev &fd, const float *
     return gi;
 }
 
+template <int SPLIT>
 __global__ void __launch_bounds__(256)
 hgrad_kernel(const FieldDev *__restrict__ fields, const ChunkItem *__restrict__ chunks, int n_chunks,
              const float *__restrict__ gbuf, float *__restrict__ grad, const float *__restrict__ params) {
-    __shared__ float part[kHgGroups][kHgPixels];
-    const int c = blockIdx.x / kHgGroups, quarter = blockIdx.x % kHgGroups;
+    constexpr int kPixels = 256 / SPLIT, kSums = kHgGroups / SPLIT;
+    __shared__ float part[SPLIT][kPixels];
+    const int c = blockIdx.x / SPLIT;
     if (c >= n_chunks) return;
     const ChunkItem ch = chunks[c];
     const FieldDev &fd = fields[ch.field];
-    if (fd.mode != 0) return;  // fields in the frequency-domain form get dL/dh from fft_hgrad_kernel
-    const int px = threadIdx.x % kHgPixels, g = threadIdx.x / kHgPixels;
-    const int q = ch.start + quarter * kHgPixels + px;
+    if (fd.mode != 0) return;  // the transform forms write their own dL/dh
+    const int px = threadIdx.x % kPixels, g = threadIdx.x / kPixels;
+    const int q = ch.start + (int)(blockIdx.x % SPLIT) * kPixels + px;
     const int f = fd.f, N = fd.N, F = fd.F, E = fd.E;
     const long long plane = (long long)f * f * N * N;
     const int ph = q / (N * N), m = q - ph * N * N;
     const int vy = f * (m / N) + ph / f, vx = f * (m % N) + ph % f;
     const int quads = E / kHgGroups * kHgGroups;
-    float acc = 0.f;
+    float acc[kSums];
+#pragma unroll
+    for (int u = 0; u < kSums; ++u) acc[u] = 0.f;
     if (q < F * F) {
         const float *Gb = gbuf + fd.gbuf_off;
         const float *dl = params + fd.param_off + (long long)F * F + (long long)E * fd.M + 2 * fd.M;
@@ -540,17 +542,26 @@ hgrad_kernel(const FieldDev *__restrict__ fields, const ChunkItem *__restrict__ 
             }
             return fd.translate ? hgrad_shifted(fd, Gi, dl + 2 * i, vx, vy) : Gi[q];
         };
-#pragma unroll 4
-        for (int i = g; i < quads; i += kHgGroups) acc += term(i);
+#pragma unroll(kHgGroups / kSums)
+        for (int i = g; i < quads; i += kHgGroups) {
+#pragma unroll
+            for (int u = 0; u < kSums; ++u) acc[u] += term(i + u);
+        }
         if (g == 0)
-            for (int i = quads; i < E; ++i) acc += term(i);
+            for (int i = quads; i < E; ++i) acc[0] += term(i);
     }
-    part[g][px] = acc;
-    __syncthreads();
-    if (g != 0 || q >= F * F) return;
+    float sum;
+    if constexpr (SPLIT == 1) {
+        sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    } else {
+        part[g][px] = acc[0];
+        __syncthreads();
+        if (g != 0) return;
+        sum = (part[0][px] + part[1][px]) + (part[2][px] + part[3][px]);
+    }
+    if (q >= F * F) return;
     const int u = vy * F + vx;
-    grad[fd.param_off + u] =
-        ((part[0][px] + part[1][px]) + (part[2][px] + part[3][px])) + fd.starlet[(long long)fd.J * F * F + u];
+    grad[fd.param_off + u] = sum + fd.starlet[(long long)fd.J * F * F + u];
 }
 
 // The moved channel's part of dL/d delta_i = f sum_u G_i(u) d(T h)(u)/d s, with d(T h)/d s_x =
@@ -830,9 +841,16 @@ void launch_psgrad(const FieldDev *fields, const int4 *ps_items, int n, const fl
         fields, ps_items, n, params, gbuf, ps_da, ps_du);
 }
 
-void launch_hgrad(const FieldDev *fields, const ChunkItem *chunks, int n_chunks, const float *gbuf, float *grad,
-                  const float *params, cudaStream_t st) {
-    hgrad_kernel<<<n_chunks * kHgGroups, 256, 0, st>>>(fields, chunks, n_chunks, gbuf, grad, params);
+// A table of few chunks is bound by the chain of each pixel's gathers over its epochs (rotated frames test 9
+// candidates per epoch) and splits them over the block, a full one loses by that: rotated fields of 24 epochs
+// of 64 x 64, us an evaluation split / not: one field (64 chunks) 200 / 229, six (384) 532 / 546, eight (512) 658 /
+// 651, 32 2128 / 2107; 32 of 10 epochs of 96 x 96 (4608) 2084 / 1955.
+void launch_hgrad(const FieldDev *fields, const ChunkItem *chunks, int n_chunks, int n_direct, int n_sms,
+                  const float *gbuf, float *grad, const float *params, cudaStream_t st) {
+    if (n_direct < 3 * n_sms)
+        hgrad_kernel<kHgGroups><<<n_chunks * kHgGroups, 256, 0, st>>>(fields, chunks, n_chunks, gbuf, grad, params);
+    else
+        hgrad_kernel<1><<<n_chunks, 256, 0, st>>>(fields, chunks, n_chunks, gbuf, grad, params);
 }
 
 void launch_hshift_grad(const FieldDev *fields, int n_fields, int E_max, int F_max, const float *params,

@@ -26,8 +26,9 @@ void launch_adj(const FieldDev *fields, const TileItem *items, int n_items, int 
                 float *gbuf, int grid, int smem, cudaStream_t st);
 void launch_psgrad(const FieldDev *fields, const int4 *ps_items, int n, const float *params, const float *gbuf,
                    float *ps_da, float *ps_du, cudaStream_t st);
-void launch_hgrad(const FieldDev *fields, const ChunkItem *chunks, int n_chunks, const float *gbuf, float *grad,
-                  const float *params, cudaStream_t st);
+// dL/dh of the direct-form fields, which n_direct of the chunks belong to
+void launch_hgrad(const FieldDev *fields, const ChunkItem *chunks, int n_chunks, int n_direct, int n_sms,
+                  const float *gbuf, float *grad, const float *params, cudaStream_t st);
 // threads of the shift gradient's block that take a field of F x F
 __host__ __device__ constexpr int hshift_threads(int F) {
     return F * F / 16 < 128 ? 128 : F * F / 16 > 1024 ? 1024 : (F * F / 16 + 31) / 32 * 32;
