@@ -10,6 +10,8 @@
 #include <functional>
 #include <map>
 #include <atomic>
+#include <iterator>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <queue>
@@ -172,19 +174,72 @@ using namespace sr;
 // buffers; the sources' gradients read the adjoint images while dL/dh is formed from them.  The owner's
 // stream orders a plan's evaluations, and both events tie the branch to it.  Not open (no stream): the
 // work stays in order on the evaluation's stream.
+//
+// A stream holds about 0.5 MB of device memory, as much as a small problem, so the plans of one owner's stream
+// share theirs: those plans' evaluations come one after another anyway (and a capture of that stream, which
+// takes its branches along, already bars any other use of it).  The events are each plan's own.  The last
+// plan of an owner's stream closes its branches.
+struct BranchStreams {
+    enum { kPrior, kPts, kSrc, kStep, kCount };
+    std::mutex m;
+    cudaStream_t s[kCount] = {};
+    ~BranchStreams() {
+        for (cudaStream_t st : s)
+            if (st) cudaStreamDestroy(st);
+    }
+    sr_status get(int k, cudaStream_t *out) {
+        std::lock_guard<std::mutex> lock(m);
+        if (!s[k]) SR_CUDA(cudaStreamCreateWithFlags(&s[k], cudaStreamNonBlocking));
+        *out = s[k];
+        return SR_OK;
+    }
+};
+
+static std::mutex g_branch_mutex;
+static std::map<std::pair<int, cudaStream_t>, std::weak_ptr<BranchStreams>> g_branches;  // by device, owner
+
+// The branches of the owner's stream on the current device; of the per-thread default stream, one name for
+// a stream of every thread, a plan has its own.
+static sr_status branch_streams(cudaStream_t owner, std::shared_ptr<BranchStreams> *out) {
+    int dev = 0;
+    SR_CUDA(cudaGetDevice(&dev));
+    std::shared_ptr<BranchStreams> set(new (std::nothrow) BranchStreams());
+    if (!set) return fail(SR_ERR_OOM, "host allocation failed");
+    if (owner != cudaStreamPerThread) {
+        std::lock_guard<std::mutex> lock(g_branch_mutex);
+        for (auto it = g_branches.begin(); it != g_branches.end();) it = it->second.expired() ? g_branches.erase(it) : std::next(it);
+        std::weak_ptr<BranchStreams> &slot = g_branches[{dev, owner}];
+        if (std::shared_ptr<BranchStreams> held = slot.lock()) set = held;
+        else slot = set;
+    }
+    *out = set;
+    return SR_OK;
+}
+
+namespace sr {
+int branch_stream_count() {  // streams that the living plans hold
+    std::lock_guard<std::mutex> lock(g_branch_mutex);
+    int n = 0;
+    for (const auto &b : g_branches)
+        if (std::shared_ptr<BranchStreams> set = b.second.lock()) {
+            std::lock_guard<std::mutex> inner(set->m);
+            for (cudaStream_t st : set->s) n += st != nullptr;
+        }
+    return n;
+}
+}  // namespace sr
+
 struct Branch {
-    cudaStream_t stream = nullptr;
+    cudaStream_t stream = nullptr;  // of the set
     cudaEvent_t forked = nullptr, joined = nullptr;
     ~Branch() {
         if (forked) cudaEventDestroy(forked);
         if (joined) cudaEventDestroy(joined);
-        if (stream) cudaStreamDestroy(stream);
     }
-    sr_status open() {
+    sr_status open(BranchStreams &set, int k) {
         if (!forked) SR_CUDA(cudaEventCreateWithFlags(&forked, cudaEventDisableTiming));
         if (!joined) SR_CUDA(cudaEventCreateWithFlags(&joined, cudaEventDisableTiming));
-        if (!stream) SR_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
-        return SR_OK;
+        return set.get(k, &stream);
     }
     // the branch's stream, ordered after everything queued on `st` so far; `st` itself when not open
     // (or when the fork fails: the order is then kept)
@@ -270,6 +325,7 @@ struct Plan {
     std::vector<cudaEvent_t> prof_ev;
     // Branches of the evaluation beside its own stream (see Branch): the starlet prior on h, the
     // point-source prior, the sources' gradients, and an optimiser step's counter
+    std::shared_ptr<BranchStreams> branches;
     Branch prior, pts, src, step;
     DevArena arena;
     ~Plan() {
@@ -518,6 +574,7 @@ struct PlanOptions {
     int grid_limit = 0;      // > 0: at most this many blocks in the persistent kernels
     int chunk = 0;           // epochs per work item of the transform form (even, <= kFftChunk; 0: by rule)
     int gp_cap = 0;          // 1: one epoch pair per group in the transform form (0: the widest compiled)
+    cudaStream_t owner = nullptr;  // the stream of the plan's evaluations
 };
 
 static bool field_uses_fft(sr_problem *p, const PlanOptions &opt);
@@ -925,9 +982,10 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
         }
     }
     if (!plain && opt.grid_limit == 0) {  // (the form autotuner times its plans in order)
-        if ((st = pl->prior.open()) != SR_OK) return st;
-        if (pl->n_sh > 0 && (st = pl->pts.open()) != SR_OK) return st;
-        if (pl->n_ps > 0 && (st = pl->src.open()) != SR_OK) return st;
+        if ((st = branch_streams(opt.owner, &pl->branches)) != SR_OK) return st;
+        if ((st = pl->prior.open(*pl->branches, BranchStreams::kPrior)) != SR_OK) return st;
+        if (pl->n_sh > 0 && (st = pl->pts.open(*pl->branches, BranchStreams::kPts)) != SR_OK) return st;
+        if (pl->n_ps > 0 && (st = pl->src.open(*pl->branches, BranchStreams::kSrc)) != SR_OK) return st;
     }
     return SR_OK;
 }
@@ -1132,7 +1190,9 @@ static sr_status ensure_plan(sr_problem *p) {
     Plan *pl = new (std::nothrow) Plan();
     if (!pl) return fail(SR_ERR_OOM, "host allocation failed");
     sr_problem *arr[1] = {p};
-    sr_status st = build_plan(pl, arr, 1, p->desc.kind == SR_DECONV && p->desc.conv_mode == SR_CONV_PLAIN);
+    PlanOptions opt;
+    opt.owner = p->stream;
+    sr_status st = build_plan(pl, arr, 1, p->desc.kind == SR_DECONV && p->desc.conv_mode == SR_CONV_PLAIN, opt);
     if (st != SR_OK) {
         delete pl;
         return st;
@@ -1148,7 +1208,7 @@ static sr_status ensure_opt_buffers(Plan *pl) {
     // a call that runs out of memory on the way leaves what it has to the next one
     for (float **p : {&pl->opt_m, &pl->opt_v, &pl->grad_int})
         if (!*p && (st = pl->arena.alloc(p, pl->n_params)) != SR_OK) return st;
-    if (!pl->plain && (st = pl->step.open()) != SR_OK) return st;
+    if (pl->branches && (st = pl->step.open(*pl->branches, BranchStreams::kStep)) != SR_OK) return st;
     SR_CUDA(cudaMemset(pl->opt_m, 0, sizeof(float) * pl->n_params));
     SR_CUDA(cudaMemset(pl->opt_v, 0, sizeof(float) * pl->n_params));
     SR_CUDA(cudaMemset(pl->d_t, 0, sizeof(long long)));
@@ -1773,7 +1833,9 @@ sr_status sr_batch_create(sr_problem *const *problems, int n, void *cuda_stream,
         delete b;
         return fail(SR_ERR_OOM, "host allocation failed");
     }
-    sr_status st = build_plan(b->plan, problems, n, false);
+    PlanOptions opt;
+    opt.owner = b->stream;
+    sr_status st = build_plan(b->plan, problems, n, false, opt);
     if (st != SR_OK) {
         delete b->plan;
         delete b;
@@ -1792,6 +1854,7 @@ static sr_status batch_replan(sr_batch *b, int chunk, int gp) {
     PlanOptions opt;
     opt.chunk = chunk;
     opt.gp_cap = gp;
+    opt.owner = b->stream;
     sr_status st = build_plan(pl, b->probs.data(), (int)b->probs.size(), false, opt);
     if (st != SR_OK) {
         delete pl;
