@@ -21,6 +21,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "lbfgsb.cuh"
+#include "once.cuh"
 
 namespace sr {
 
@@ -104,39 +105,39 @@ struct DevArena {
     ~DevArena() { release(); }
 };
 
-static int g_smem_optin = -1;
-static int g_num_sms = 0;
-static int g_fft_smem_limit = 0;  // dynamic shared memory the transform kernels can take
-static int g_fx_smem_limit = 0;   // ... and the per-epoch chunk kernel
+// Of the devices set up so far, the smallest (plans are sized for any of them).
+static std::atomic<int> g_smem_optin{-1};
+static std::atomic<int> g_num_sms{0};
+static std::atomic<int> g_fft_smem_limit{0};  // dynamic shared memory the transform kernels can take
+static std::atomic<int> g_fx_smem_limit{0};   // ... and the per-epoch chunk kernel
 
-// The limits are published (g_dev_ready, set last) only once every kernel is configured; host
-// threads making their first calls together configure once, under the lock.
-static std::mutex g_dev_mutex;
-static std::atomic<bool> g_dev_ready{false};
+// The kernels' shared-memory limits and constant tables belong to a device, so each is configured at its
+// first use.  Limits narrow before the device counts as ready.
+static OncePerDevice g_dev_once;
 
 static sr_status device_limits() {
-    if (g_dev_ready.load(std::memory_order_acquire)) return SR_OK;
-    std::lock_guard<std::mutex> lock(g_dev_mutex);
-    if (g_dev_ready.load(std::memory_order_relaxed)) return SR_OK;
-    int dev = 0, optin = 0, sms = 0;
-    SR_CUDA(cudaGetDevice(&dev));
-    SR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    SR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // reserve the static shared memory of the tile kernels
-    const int dyn = optin - kTileStaticReserve;
-    sr_status s = configure_tile_kernels(dyn, dyn);
-    if (s != SR_OK) return s;
-    int fx = 0, fft = 0;
-    s = configure_fft_pair(optin, &fx, &fft);
-    if (s != SR_OK) return s;
-    s = configure_fft_big(optin);
-    if (s != SR_OK) return s;
-    g_smem_optin = optin;
-    g_num_sms = sms;
-    g_fx_smem_limit = fx;
-    g_fft_smem_limit = fft;
-    g_dev_ready.store(true, std::memory_order_release);
-    return SR_OK;
+    return g_dev_once.run([]() -> sr_status {
+        int dev = 0, optin = 0, sms = 0;
+        SR_CUDA(cudaGetDevice(&dev));
+        SR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        SR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        // reserve the static shared memory of the tile kernels
+        const int dyn = optin - kTileStaticReserve;
+        sr_status s = configure_tile_kernels(dyn, dyn);
+        if (s != SR_OK) return s;
+        int fx = 0, fft = 0;
+        s = configure_fft_pair(optin, &fx, &fft);
+        if (s != SR_OK) return s;
+        s = configure_fft_big(optin);
+        if (s != SR_OK) return s;
+        const bool first = g_num_sms == 0;
+        auto narrow = [&](std::atomic<int> &limit, int v) { limit = first ? v : std::min(limit.load(), v); };
+        narrow(g_smem_optin, optin);
+        narrow(g_fx_smem_limit, fx);
+        narrow(g_fft_smem_limit, fft);
+        narrow(g_num_sms, sms);
+        return SR_OK;
+    });
 }
 
 // Transform size for the frequency-domain form: the smallest listed L (the sizes the transform
@@ -595,7 +596,7 @@ static int default_chunk(sr_problem *const *probs, int n, int epoch_limit) {
         int epochs, group;
     };
     std::vector<Shape> sh;
-    const int sms = std::max(g_num_sms, 1);
+    const int sms = std::max(g_num_sms.load(), 1);
     long long longest = 0;
     for (int i = 0; i < n; ++i) {
         const sr_problem *p = probs[i];

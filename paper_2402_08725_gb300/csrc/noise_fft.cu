@@ -19,7 +19,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <atomic>
 #include <complex>
 #include <mutex>
 
@@ -27,6 +26,7 @@
 #include "cplx.cuh"
 #include "fft_pair.cuh"
 #include "noise.cuh"
+#include "once.cuh"
 
 namespace sr {
 namespace {
@@ -148,15 +148,11 @@ sr_status nf_block(Kern kernel, int smem, int *threads, int *occ) {
 
 // the DFT twiddles of this translation unit, once per device
 sr_status nf_tables() {
-    static std::mutex m;
-    static bool done[64] = {};
-    int dev = 0;
-    SR_CUDA(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lock(m);
-    if (dev < 64 && done[dev]) return SR_OK;
-    SR_CUDA(pr_fill_dtw());
-    if (dev < 64) done[dev] = true;
-    return SR_OK;
+    static OncePerDevice once;
+    return once.run([]() -> sr_status {
+        SR_CUDA(pr_fill_dtw());
+        return SR_OK;
+    });
 }
 
 // The in-register DFTs of fft_pair.cuh (dft<R, false>) in FP64 with the same FP32 constants: v[k] in,

@@ -31,11 +31,11 @@
 // Fields deeper than a level skip it.
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "common.cuh"
 #include "ffsum.cuh"
 #include "kernels.cuh"
+#include "once.cuh"
 
 namespace sr {
 
@@ -712,15 +712,9 @@ int starlet_comb_rows_bits(const int *F, const int *J, int n, int n_sms) {
 
 int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, const ChunkItem *chunks,
                    int n_chunks, int Jmax, const float *params, double *l1_part, cudaStream_t st) {
-    // the kernels' budgets of dynamic shared memory, once per device (host threads evaluating at once
-    // wait for whichever configures it)
-    static std::mutex config_mutex;
-    static std::atomic<unsigned long long> configured{0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (!(configured.load(std::memory_order_acquire) & bit)) {
-        std::lock_guard<std::mutex> lock(config_mutex);
+    // the kernels' budgets of dynamic shared memory
+    static OncePerDevice configured;
+    configured.run([]() -> sr_status {
         cudaFuncSetAttribute(starlet_band_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
         cudaFuncSetAttribute(starlet_band_adj_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
         cudaFuncSetAttribute(starlet_tile_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes);
@@ -735,8 +729,8 @@ int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, co
         cudaFuncSetAttribute(starlet_comb_adj_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
         cudaFuncSetAttribute(starlet_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
         cudaFuncSetAttribute(starlet_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemBytes);
-        configured.fetch_or(bit, std::memory_order_release);
-    }
+        return SR_OK;
+    });
     const bool bands = (forms & 1) != 0, tiles = (forms & 2) != 0;
     const bool map = (forms & kStarletMapBit) != 0;
     // comb-band fields: in clusters up to kClusterMaxF when the table asks for it, the others (if any)

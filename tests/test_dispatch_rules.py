@@ -1,14 +1,15 @@
 """The host's rules that choose a kernel, a tile or a schedule, on the CPU."""
 import ctypes
+import os
 import subprocess
 
 from paper_2402_08725_gb300 import build
 
 
-def _run_cpp(tmp_path, body):
+def _run_cpp(tmp_path, body, head='#include "kernels.cuh"\n'):
     """Integers printed by the statements `body`, compiled against the library's internal headers."""
     src, exe = tmp_path / "rule.cu", str(tmp_path / "rule")
-    src.write_text('#include <cstdio>\n#include "kernels.cuh"\nint main() {\n' + body + "\n}\n")
+    src.write_text("#include <cstdio>\n" + head + "int main() {\n" + body + "\n}\n")
     subprocess.run([build.nvcc(), "-std=c++17", "-I", build.INCLUDE, "-I", build.CSRC, str(src), "-o", exe], check=True)
     return [int(v) for v in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()]
 
@@ -54,3 +55,36 @@ def test_shift_gradient_threads_follow_the_grid(tmp_path):
     """About 16 pixels a thread, whole warps, 128 to 1024 threads."""
     got = _run_cpp(tmp_path, "".join(f'  printf("%d\\n", sr::hshift_threads({F}));\n' for F in (5, 64, 90, 128, 1536)))
     assert got == [128, 256, 512, 1024, 1024]
+
+
+def test_each_device_is_set_up_once(tmp_path):
+    """A second device gets its own set-up, a failed one is repeated, and threads together run it once."""
+    head = """#include <atomic>
+#include <thread>
+#include <vector>
+#include "once.cuh"
+namespace sr { sr_status cuda_fail(cudaError_t, const char *) { return SR_ERR_CUDA; } }
+"""
+    body = """
+  sr::OncePerDevice once;
+  std::atomic<int> n{0};
+  auto ok = [&] { ++n; return SR_OK; };
+  auto bad = [&] { ++n; return SR_ERR_CUDA; };
+  printf("%d ", (int)once.run_on(0, bad));
+  once.run_on(0, ok); once.run_on(0, ok); printf("%d ", n.load());   // failed, then done once
+  once.run_on(1, ok); once.run_on(1, ok); printf("%d ", n.load());   // another device
+  once.run_on(63, ok); once.run_on(63, ok); once.run_on(64, ok); once.run_on(64, ok); printf("%d ", n.load());
+  std::vector<std::thread> t;
+  for (int k = 0; k < 8; ++k) t.emplace_back([&] { once.run_on(2, ok); });
+  for (auto &x : t) x.join();
+  printf("%d", n.load());
+"""
+    assert _run_cpp(tmp_path, body, head) == [4, 2, 3, 6, 7]
+
+
+def test_the_kernels_of_every_file_are_set_up_per_device():
+    """No kernel attribute or constant table is set behind a once-per-process flag."""
+    for name in sorted(os.listdir(build.CSRC)):
+        with open(os.path.join(build.CSRC, name)) as fh:
+            text = fh.read()
+        assert "once_flag" not in text and "static std::atomic<bool>" not in text, name
