@@ -678,7 +678,7 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
                 Es.push_back(opt.epoch_limit > 0 ? std::min(probs[i]->desc.n_epochs, opt.epoch_limit) : probs[i]->desc.n_epochs);
                 Ns.push_back(probs[i]->desc.data_n);
             }
-        rows = tile_rows(Es.data(), Ns.data(), (int)Es.size(), g_num_sms);
+        rows = tile_rows(Es.data(), Ns.data(), (int)Es.size(), g_num_sms, opt.grid_limit);
     }
     for (int i = 0; i < n; ++i) {
         sr_problem *p = probs[i];

@@ -801,8 +801,10 @@ int choose_tile_pg(int nph, TileItem t, int Tk, int smem_limit) {
 // (64 rows) or one (32).  Rotated fields of 24 epochs of 64 x 64, us an evaluation with 64 / 32 / 16 rows: one
 // field (24 items of 64 rows) 407 / 268 / 203, four 463 / 426 / 409, eight 733 / 661 / 701, sixteen 1138 / 1167 /
 // 1233, 32 2125 / 2166 / 2389; of 10 epochs of 96 x 96, eight (320 items of 64) 890 / 691 / 722, sixteen 1186 /
-// 1197 / 1321.  The results do not depend on it.
-int tile_rows(const int *E, const int *N, int n, int n_sms) {
+// 1197 / 1321.  The results do not depend on it.  The form autotuner, which times a field's first epochs on one
+// block (grid_limit) for the batches that fill the GPU, times the tiles those take.
+int tile_rows(const int *E, const int *N, int n, int n_sms, int grid_limit) {
+    if (grid_limit > 0) return 64;
     for (int rows : {64, 32}) {
         long long items = 0;
         for (int i = 0; i < n; ++i) items += (long long)E[i] * ((N[i] + 63) / 64) * ((N[i] + rows - 1) / rows);

@@ -15,8 +15,9 @@ constexpr int kTileStaticReserve = 2048;
 void launch_kappa_prep(const float *s, float *kappa, int E, int K, int f, int Tk, int tau_lo, cudaStream_t st);
 int tile_smem_bytes(const TileItem &t, int Tk, bool fwd);
 // phase groups of a tile: the most (a divisor of f^2) that fit one block and smem_limit bytes
-// Rows of the direct form's output tiles (64, 32 or 16) for a table of n direct fields of E epochs of N x N.
-int tile_rows(const int *E, const int *N, int n, int n_sms);
+// Rows of the direct form's output tiles (64, 32 or 16) for a table of n direct fields of E epochs of N x N, run
+// on at most grid_limit blocks (0: on all that fit).
+int tile_rows(const int *E, const int *N, int n, int n_sms, int grid_limit);
 int choose_tile_pg(int nph, TileItem t, int Tk, int smem_limit);
 sr_status configure_tile_kernels(int smem_fwd, int smem_adj);
 sr_status occupancy_tile_kernels(int smem_fwd, int smem_adj, int *blocks_fwd, int *blocks_adj);

@@ -33,11 +33,17 @@ def _ints(v):
 def test_tile_height_is_the_tables():
     """A field that leaves SMs idle alone takes short tiles; the same field in a batch that fills them does not
     pay their halo."""
-    rows = _rule("_ZN2sr9tile_rowsEPKiS1_ii")
+    rows = _rule("_ZN2sr9tile_rowsEPKiS1_iii")
     for n, want in ((1, 16), (4, 16), (8, 32), (16, 32), (32, 64)):
-        assert rows(_ints([24] * n), _ints([64] * n), n, 152) == want
-    assert rows(_ints([300]), _ints([64]), 1, 152) == 32
-    assert rows(_ints([]), _ints([]), 0, 152) == 16
+        assert rows(_ints([24] * n), _ints([64] * n), n, 152, 0) == want
+    assert rows(_ints([300]), _ints([64]), 1, 152, 0) == 32
+    assert rows(_ints([]), _ints([]), 0, 152, 0) == 16
+
+
+def test_the_form_autotuner_times_the_tiles_of_full_batches():
+    """Its verdict is kept by shape, for any number of epochs: the first field's must not enter it."""
+    rows = _rule("_ZN2sr9tile_rowsEPKiS1_iii")
+    assert {rows(_ints([E]), _ints([64]), 1, 152, 1) for E in (1, 4, 16)} == {64}
 
 
 def test_clusters_only_where_they_run_at_once():

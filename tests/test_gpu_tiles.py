@@ -15,7 +15,7 @@ def _rows(E, N, n):
     from paper_2402_08725_gb300 import _native
     lib = ctypes.CDLL(_native.load()._name)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    return lib._ZN2sr9tile_rowsEPKiS1_ii((ctypes.c_int * n)(*[E] * n), (ctypes.c_int * n)(*[N] * n), n, sms)
+    return lib._ZN2sr9tile_rowsEPKiS1_iii((ctypes.c_int * n)(*[E] * n), (ctypes.c_int * n)(*[N] * n), n, sms, 0)
 
 
 @pytest.mark.parametrize("frame", ["plain", "shifted", "rotated"])
