@@ -7,14 +7,12 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <functional>
 #include <map>
 #include <atomic>
 #include <iterator>
 #include <memory>
 #include <mutex>
 #include <new>
-#include <queue>
 #include <string>
 #include <vector>
 
@@ -580,65 +578,17 @@ struct PlanOptions {
 
 static bool field_uses_fft(sr_problem *p, const PlanOptions &opt);
 
-// Default epochs per work item of the transform form (even, 2 .. kFftChunk): the shortest time to
-// finish the items on one block per SM, longest first, plus the traffic of their accumulators.
-// An item costs its epoch pairs' transforms (measured: 8 to 11 cycles per point of the L x L pair at
-// f = 2, by the phases above that, and 0.45 more per further source; 0.6 of it once per group of pairs,
-// whose passes it shares) and a fixed part; an accumulator is written, read back and added at about
-// 400 bytes a clock over the GPU.  Against "as many epochs as keep
-// two items per SM" (us per evaluation): 1000 epochs of 32 x 32 157 -> 102 (8 epochs instead of 2: 125
-// items finish together, 500 leave a fourth of a round and 4 times the accumulators), 500 of 48 x 48
-// 123 -> 94, 24 fields of 10-60 epochs 269 -> 193; 300 of 64 x 64 keeps 2.  Fields that fill the GPU several
-// times at the longest items take those.
-static int default_chunk(sr_problem *const *probs, int n, int epoch_limit) {
-    struct Shape {
-        double pair, acc;  // cycles of a pair; accumulator bytes
-        int epochs, group;
-    };
-    std::vector<Shape> sh;
-    const int sms = std::max(g_num_sms.load(), 1);
-    long long longest = 0;
+// Default epochs per work item of the transform form for these problems (fft_chunk_epochs).
+static int default_chunk(sr_problem *const *probs, int n, const PlanOptions &opt) {
+    std::vector<FftShape> sh;
     for (int i = 0; i < n; ++i) {
         const sr_problem *p = probs[i];
         if (!p->fft_ok || p->fft_big) continue;
-        const double L = p->fft_L, nph = (double)p->desc.supersampling * p->desc.supersampling;
-        const int E = epoch_limit > 0 ? std::min(p->desc.n_epochs, epoch_limit) : p->desc.n_epochs;
-        sh.push_back({9.0 * L * L * (0.25 + 0.1875 * nph) * (1.0 + 0.45 * std::max(0, p->desc.n_sources - 1)),
-                      nph * L * (L / 2 + 2) * 8.0, E, fft_pair_gpmax(p->fft_L, p->desc.n_sources)});
-        longest += (E + kFftChunk - 1) / kFftChunk;
+        const sr_problem_desc &d = p->desc;
+        sh.push_back({p->fft_L, d.n_sources, d.supersampling,
+                      opt.epoch_limit > 0 ? std::min(d.n_epochs, opt.epoch_limit) : d.n_epochs});
     }
-    if (longest >= 4LL * sms) return kFftChunk;
-    std::stable_sort(sh.begin(), sh.end(), [](const Shape &a, const Shape &b) { return a.pair > b.pair; });
-    int best = 2;
-    double best_t = 0.0;
-    for (int c = 2; c <= kFftChunk; c += 2) {
-        std::vector<double> items;
-        double bytes = 0.0;
-        for (const Shape &s : sh)
-            for (int e = 0; e < s.epochs; e += c) {
-                const int pairs = (std::min(c, s.epochs - e) + 1) / 2, groups = (pairs + s.group - 1) / s.group;
-                items.push_back((0.6 * groups + 0.4 * pairs) * s.pair + 4000.0);
-                bytes += 2.0 * s.acc;
-            }
-        std::sort(items.begin(), items.end(), [](double a, double b) { return a > b; });
-        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-        double end = 0.0;
-        for (double t : items) {
-            double at = 0.0;
-            if ((int)free_at.size() >= sms) {
-                at = free_at.top();
-                free_at.pop();
-            }
-            free_at.push(at + t);
-            end = std::max(end, at + t);
-        }
-        const double total = end + bytes / 400.0;
-        if (c == 2 || total < std::min(0.95 * best_t, best_t - 20000.0)) {  // 10 us at least
-            best = c;
-            best_t = total;
-        }
-    }
-    return best;
+    return fft_chunk_epochs(sh.data(), (int)sh.size(), std::max(g_num_sms.load(), 1), g_fx_smem_limit);
 }
 
 // Build the evaluation plan of `n` problems of the same kind.
@@ -666,7 +616,7 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
     std::vector<ChunkItem> sh_chunks;
     long long pbar_len = 0, l1pts = 0, ptsslot = 0;
     long long hs_len = 0;
-    int chunk = opt.chunk > 0 ? opt.chunk : default_chunk(probs, n, opt.epoch_limit);
+    int chunk = opt.chunk > 0 ? opt.chunk : default_chunk(probs, n, opt);
     chunk = std::max(2, std::min(kFftChunk, chunk)) & ~1;
     pl->chunk = chunk;
     pl->gp_cap = opt.gp_cap;
@@ -747,10 +697,7 @@ static sr_status build_plan(Plan *pl, sr_problem *const *probs, int n, bool plai
             pl->max_pairs = std::max(pl->max_pairs, (nph + 1) / 2);
             pl->max_acc_points = std::max(pl->max_acc_points, nph * fd.fft_L * (fd.fft_L / 2 + 1));
             smem_fft = std::max(smem_fft, fft_pair_field_smem(L));
-            // epoch pairs side by side: the widest group the kernel is compiled for at this size
-            // (more than one pair only with at most one source) if its buffers fit, else one pair
-            int G = opt.gp_cap != 1 ? fft_pair_gpmax(L, fd.M) : 1;
-            if (G > 1 && fft_pair_smem_bytes(L, fd.M, fd.f, G) > g_fx_smem_limit) G = 1;
+            const int G = fft_pair_group(L, fd.M, fd.f, opt.gp_cap, g_fx_smem_limit);
             fd.fft_G = G;
             smem_fx = std::max(smem_fx, fft_pair_smem_bytes(L, fd.M, fd.f, G));
         } else if (pl->kind == SR_DECONV && !plain) {

@@ -44,6 +44,9 @@
 #include <math.h>
 
 #include <algorithm>
+#include <functional>
+#include <queue>
+#include <vector>
 
 #include "common.cuh"
 #include "cplx.cuh"
@@ -730,6 +733,72 @@ int fft_pair_gpmax(int L, int M) {
         default:
             return 1;
     }
+}
+
+// Epoch pairs side by side: the widest group the kernel is compiled for at this size (more than one pair
+// only with at most one source) if its buffers fit, else one pair.
+int fft_pair_group(int L, int M, int f, int gp_cap, int smem_limit) {
+    const int G = gp_cap != 1 ? fft_pair_gpmax(L, M) : 1;
+    return G > 1 && fft_pair_smem_bytes(L, M, f, G) > smem_limit ? 1 : G;
+}
+
+// Default epochs per work item of the transform form (even, 2 .. kFftChunk): the shortest time to
+// finish the items on one block per SM, longest first, plus the traffic of their accumulators.
+// An item costs its epoch pairs' transforms (measured: 8 to 11 cycles per point of the L x L pair at
+// f = 2, by the phases above that, and 0.45 more per further source; 0.6 of it once per group of pairs,
+// whose passes it shares) and a fixed part; an accumulator is written, read back and added at about
+// 400 bytes a clock over the GPU.  Against "as many epochs as keep two items per SM" (us per evaluation):
+// 1000 epochs of 32 x 32 157 -> 102 (8 epochs instead of 2: 125 items finish together, 500 leave a fourth of
+// a round and 4 times the accumulators), 500 of 48 x 48 123 -> 94, 24 fields of 10-60 epochs 269 -> 193; 300 of 64 x 64 keeps 2, 300 of 88 x 88 at f =
+// 3, whose buffers leave room for one pair, take 2 (193; 222 with the 4 of two pairs).  Groups capped to one pair by
+// the caller keep the epochs of the widest (1000 of 24 x 24: 104 with 8, 126 with the 4 of that pricing).  Fields
+// that fill the GPU several times at the longest items take those.
+int fft_chunk_epochs(const FftShape *shapes, int n, int n_sms, int smem_limit) {
+    struct Shape {
+        double pair, acc;  // cycles of a pair; accumulator bytes
+        int epochs, group;
+    };
+    std::vector<Shape> sh;
+    long long longest = 0;
+    for (int i = 0; i < n; ++i) {
+        const FftShape &p = shapes[i];
+        const double L = p.L, nph = (double)p.f * p.f;
+        sh.push_back({9.0 * L * L * (0.25 + 0.1875 * nph) * (1.0 + 0.45 * std::max(0, p.M - 1)),
+                      nph * L * (L / 2 + 2) * 8.0, p.E, fft_pair_group(p.L, p.M, p.f, 0, smem_limit)});
+        longest += (p.E + kFftChunk - 1) / kFftChunk;
+    }
+    if (longest >= 4LL * n_sms) return kFftChunk;
+    std::stable_sort(sh.begin(), sh.end(), [](const Shape &a, const Shape &b) { return a.pair > b.pair; });
+    int best = 2;
+    double best_t = 0.0;
+    for (int c = 2; c <= kFftChunk; c += 2) {
+        std::vector<double> items;
+        double bytes = 0.0;
+        for (const Shape &s : sh)
+            for (int e = 0; e < s.epochs; e += c) {
+                const int pairs = (std::min(c, s.epochs - e) + 1) / 2, groups = (pairs + s.group - 1) / s.group;
+                items.push_back((0.6 * groups + 0.4 * pairs) * s.pair + 4000.0);
+                bytes += 2.0 * s.acc;
+            }
+        std::sort(items.begin(), items.end(), [](double a, double b) { return a > b; });
+        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+        double end = 0.0;
+        for (double t : items) {
+            double at = 0.0;
+            if ((int)free_at.size() >= n_sms) {
+                at = free_at.top();
+                free_at.pop();
+            }
+            free_at.push(at + t);
+            end = std::max(end, at + t);
+        }
+        const double total = end + bytes / 400.0;
+        if (c == 2 || total < std::min(0.95 * best_t, best_t - 20000.0)) {  // 10 us at least
+            best = c;
+            best_t = total;
+        }
+    }
+    return best;
 }
 
 // Whether the chunk kernel takes M sources at size L (one pair per group, two phases).

@@ -57,7 +57,14 @@ int fft_pair_zn(int L);       // float2 elements of one pair array
 int fft_pair_smem_bytes(int L, int M, int f, int GP);  // chunk kernel, GP epoch pairs per group
 int fft_pair_field_smem(int L);                        // per-field and per-PSF kernels
 bool fft_pair_variant(int L, int M);                   // the chunk kernel takes M sources at this size
-int fft_pair_gpmax(int L, int M);                      // epoch pairs per group
+int fft_pair_gpmax(int L, int M);                      // most epoch pairs per group
+// epoch pairs per group of a field (gp_cap 1: one; else the most whose buffers fit smem_limit)
+int fft_pair_group(int L, int M, int f, int gp_cap, int smem_limit);
+struct FftShape {
+    int L, M, f, E;
+};
+// default epochs per work item of the transform form for a table of n such fields (even, 2 .. kFftChunk)
+int fft_chunk_epochs(const FftShape *shapes, int n, int n_sms, int smem_limit);
 sr_status configure_fft_pair(int optin, int *chunk_limit, int *field_limit);
 sr_status configure_fft_pair_field(int optin, int *field_limit);  // called by configure_fft_pair
 // spectra of a problem's folded kernels (set_psfs): [ceil(E/2)][f*f][L][L/2+2] of (re_a, re_b, im_a,

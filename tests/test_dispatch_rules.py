@@ -94,3 +94,17 @@ def test_the_kernels_of_every_file_are_set_up_per_device():
         with open(os.path.join(build.CSRC, name)) as fh:
             text = fh.read()
         assert "once_flag" not in text and "static std::atomic<bool>" not in text, name
+
+
+def test_items_are_priced_by_the_groups_they_run_in():
+    """Epochs per item: where nine phases leave no room for two pairs the pairs of an item share no passes."""
+    epochs, group = _rule("_ZN2sr16fft_chunk_epochsEPKNS_8FftShapeEiii"), _rule("_ZN2sr14fft_pair_groupEiiiii")
+    limit = 229500
+
+    def item(L, M, f, E):
+        return epochs(_ints([L, M, f, E]), 1, 152, limit)
+
+    assert group(112, 1, 2, 0, limit) == 2 and group(112, 1, 3, 0, limit) == 1 and group(112, 1, 2, 1, limit) == 1
+    assert group(32, 1, 2, 0, limit) == 4 and group(32, 2, 2, 0, limit) == 1
+    assert item(112, 1, 2, 300) == 4 and item(112, 1, 3, 300) == 2 and item(32, 1, 2, 1000) == 8
+    assert epochs(_ints([]), 0, 152, limit) == 2
