@@ -273,10 +273,10 @@ __host__ __device__ constexpr int pr_r1(int L) {
     return L == 24 ? 8 : L == 32 ? 8 : L == 40 ? 8 : L == 48 ? 16 : L == 56 ? 8 : L == 64 ? 16 : L == 72 ? 8 : L == 80 ? 16 : L == 96 ? 16
          : L == 112 ? 16 : L == 128 ? 16 : L == 144 ? 16 : L == 160 ? 16 : 0;
 }
-// extra float2 per row beyond R1 S: the row pitch is brought to R2 (mod 16), except at L = 80,
-// whose four-pair groups fit in shared memory only without it, and at L = 160 (one pair does)
+// extra float2 per row beyond R1 S: the row pitch is brought to R2 (mod 16), except at L = 160, which fits in
+// shared memory only without it
 __host__ __device__ constexpr int pr_pad(int L, int RW, int R2) {
-    return L == 80 || L == 160 ? 0 : (((R2 - RW) % 16) + 16) % 16;
+    return L == 160 ? 0 : (((R2 - RW) % 16) + 16) % 16;
 }
 
 template <int L>
