@@ -1,8 +1,8 @@
-// Packed FP32 pairs and in-register DFTs over two value types (internal, device code).
+// Packed FP32 pairs and the arithmetic of in-register DFTs over two value types (internal, device code).
 //
 // sm_103a issues add, multiply and fused multiply-add on two FP32 values per instruction
 // (add/mul/fma.rn.f32x2).  The rate of the FP32 pipe is the same (78.7 against 77.2 TFLOP/s measured),
-// but half the instructions are issued, which is what bounds the chunk kernel.  The DFTs below run on
+// but half the instructions are issued, which is what bounds the chunk kernel.  zdft of fft_pair.cuh runs on
 //   float2  one complex value (x = real, y = imaginary): additions are packed;
 //   C2      two complex values side by side (the same position of two epochs): every operation is.
 #pragma once

@@ -16,7 +16,7 @@
 //   kappa_prep_kernel   folded polyphase kernels, once per set_psfs
 //   fwd_kernel<R>       persistent over (field, epoch, tile): stage F_phi tiles of h plus the
 //                       rasterised point sources in shared memory, accumulate M over all phases,
-//                       residual, FP64 chi^2 and sum(e) partials (warp shuffles), write e
+//                       residual, chi^2 and sum(e) per band of 16 rows, write e
 //   adj_kernel<R>       persistent over (field, epoch, tile): stage the e tile once, correlate
 //                       with each phase's kernel, write G_{i,phi} (per-epoch images)
 //   psgrad_kernel       per (epoch, source): <G_i, g>, <G_i, grad g> on the source window
@@ -645,15 +645,14 @@ l1_sum_kernel(const FieldDev *__restrict__ fields, const double *__restrict__ l1
 // Per-field assembly of the loss and the small parameter blocks, in fixed order.  One block per field;
 // with one field it also writes the total.  More threads do not help: the FP64 sums run at 2 additions
 // a clock per SM (37 epochs 9.8 us with 256 threads, 17.5 with 1024).
-constexpr int kFinThreads = kThreads;
-__global__ void __launch_bounds__(kFinThreads)
+__global__ void __launch_bounds__(kThreads)
 finalize_kernel(const FieldDev *__restrict__ fields, const double *__restrict__ chi_part,
                 const double *__restrict__ se_part, const double *__restrict__ l1_part,
                 const float *__restrict__ ps_da, const float *__restrict__ ps_du, float *__restrict__ grad,
                 double *__restrict__ losses, const FieldDev *__restrict__ pts_fields,
                 const double *__restrict__ l1_pts, const float *__restrict__ pts_g, const float *__restrict__ hs,
                 double *__restrict__ total, const double *__restrict__ l1_sum) {
-    __shared__ double s_red[2][kFinThreads / 32];
+    __shared__ double s_red[2][kThreads / 32];
     const FieldDev &fd = fields[blockIdx.x];
     const int E = fd.E, M = fd.M, F = fd.F, f = fd.f;
     // point-source prior of the field (Eq. 11, third term), if it has one
@@ -868,7 +867,7 @@ int launch_finalize(const FieldDev *fields, int n_fields, const double *chi_part
                     const double *l1_part, const float *ps_da, const float *ps_du, float *grad, double *losses,
                     double *total, cudaStream_t st, const FieldDev *pts_fields, const double *l1_pts,
                     const float *pts_g, const float *hs, const double *l1_sum) {
-    finalize_kernel<<<n_fields, kFinThreads, 0, st>>>(fields, chi_part, se_part, l1_part, ps_da, ps_du, grad, losses,
+    finalize_kernel<<<n_fields, kThreads, 0, st>>>(fields, chi_part, se_part, l1_part, ps_da, ps_du, grad, losses,
                                                       pts_fields, l1_pts, pts_g, hs, total, l1_sum);
     if (n_fields == 1) return 1;
     total_kernel<<<1, 32, 0, st>>>(losses, n_fields, total);

@@ -1,7 +1,7 @@
 // Per-PSF and per-field transforms of the frequency-domain form (sm_103a): the spectra of the
 // folded PSF kernels (at set_psfs), the spectra of the phase images of h (once per evaluation and
 // field) and the transform back of the accumulated adjoint spectra (dL/dh).  Each block transforms
-// two phases at once as one complex image (fft_pair.cuh).
+// two phases at once as one complex image (fft_pair.cuh), the PSF kernels two epochs of a phase.
 #include <math.h>
 
 #include <algorithm>

@@ -30,8 +30,7 @@ __device__ __forceinline__ double strided_sum4(const double *__restrict__ v, lon
 }
 
 // Deterministic block sum of two doubles (fixed shuffle tree, warps summed in order).
-template <int NW>
-__device__ __forceinline__ void block_sum2(double &a, double &b, double (*red)[NW]) {
+__device__ __forceinline__ void block_sum2(double &a, double &b, double (*red)[kThreads / 32]) {
     a = warp_sum(a);
     b = warp_sum(b);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -48,27 +47,6 @@ __device__ __forceinline__ void block_sum2(double &a, double &b, double (*red)[N
         }
         a = sa;
         b = sb;
-    }
-}
-
-// The same over compensated FP32 pairs (FP64 only for the two results, on thread 0).
-__device__ __forceinline__ void block_fsum2(FSum a, FSum b, float2 (*red)[kThreads / 32], double &oa, double &ob) {
-    a = fsum_warp(a);
-    b = fsum_warp(b);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[0][wid] = make_float2(a.hi, a.lo);
-        red[1][wid] = make_float2(b.hi, b.lo);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        FSum sa = fsum_zero(), sb = fsum_zero();
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-            sa = fsum_add(sa, FSum{red[0][i].x, red[0][i].y});
-            sb = fsum_add(sb, FSum{red[1][i].x, red[1][i].y});
-        }
-        oa = fsum_value(sa);
-        ob = fsum_value(sb);
     }
 }
 
