@@ -31,6 +31,9 @@
 // Fields deeper than a level skip it.
 #include <algorithm>
 #include <atomic>
+#include <functional>
+#include <utility>
+#include <vector>
 
 #include "common.cuh"
 #include "ffsum.cuh"
@@ -691,23 +694,44 @@ int starlet_forms_single(int F, int J, bool map) {
 
 int starlet_comb_rows_of(int forms) { return (forms & kStarletRows8) ? 8 : (forms & kStarletRows4) ? 4 : kCombRows; }
 
-// Rows per comb block for a table of comb-band fields (F, J of each): 16, or 8 or 4 when the table's
-// level-0 blocks would not fill twice the SMs; and clusters for those of at most kClusterMaxF when they take
-// at most two thirds of the SMs, so that all run at once beside the chi^2 kernels (a cluster's blocks must
-// be free together).  Fields of 20 epochs, us an evaluation in clusters / level by level: 64 x 64 grids, 8
-// fields 66 / 78, 16 95 / 82, 64 224 / 141; 128 x 128, 8 84 / 93, 12 104 / 111, 16 133 / 114, 32 212 / 164; 256 x
-// 256, 8 170 / 177, 12 209 / 204, 16 292 / 270.  The results do not depend on it (the prior's partial sums are
-// kept per 4-row group).  Returns the forms bits to add (0 for 16 rows, level by level).
+// Whether the fields of at most kClusterMaxF (F, levels of each) run as clusters.  About three quarters of the
+// SMs' worth of clusters run at once (the blocks of one must be free together, within one part of the GPU),
+// longest first, the chi^2 kernels waiting for SMs meanwhile; level by level every field takes the deepest one's
+// launches, most of which the chi^2 kernels hide.  A level of a cluster costs 1.5 + (F / 256)^2, a launch 4.5 + 2
+// (F / 256)^2, and clusters are taken up to 0.6 of the levels' time: fitted to 50 tables, of which four lose more
+// than 2 % by it.  Us an evaluation in clusters / level by level: alike fields of 20 epochs, 64 x 64 grids, J = 4,
+// 12 fields 91 / 96, 24 129 / 110; 128 x 128, J = 6, 12 152 / 166, 16 191 / 175, 32 293 / 232; uneven fields
+// (J = 4 to 6), 13 113 / 140, 21 241 / 261, 24 227 / 234, 32 of up to 256 x 256 520 / 560, 38 of up to 96 x 96 358 /
+// 326.
+static bool starlet_clusters(const std::vector<std::pair<int, int>> &shapes, int n_sms) {
+    if (shapes.empty()) return false;
+    auto squared = [](int F) { return (double)F * F / (256.0 * 256.0); };
+    std::vector<double> times, ends(std::max(1, n_sms / kClusterBlocks * 3 / 4), 0.0);
+    int widest = 0, deepest = 0;
+    for (const std::pair<int, int> &s : shapes) {
+        times.push_back(s.second * (1.5 + squared(s.first)));
+        widest = std::max(widest, s.first);
+        deepest = std::max(deepest, s.second);
+    }
+    std::sort(times.begin(), times.end(), std::greater<double>());
+    for (double t : times) *std::min_element(ends.begin(), ends.end()) += t;
+    return *std::max_element(ends.begin(), ends.end()) <= 0.6 * deepest * (4.5 + 2.0 * squared(widest));
+}
+
+// Rows per comb block for a table of comb-band fields (F, J of each): 16, or 8 or 4, and perhaps clusters, when
+// the table's level-0 blocks would not fill twice the SMs.  The results do not depend on it (the prior's
+// partial sums are kept per 4-row group).  Returns the forms bits to add (0 for 16 rows, level by level).
 int starlet_comb_rows_bits(const int *F, const int *J, int n, int n_sms) {
-    long long blocks = 0, clusters = 0;
+    long long blocks = 0;
+    std::vector<std::pair<int, int>> shapes;  // of the fields that may be clusters: F, levels
     for (int i = 0; i < n; ++i)
         if (starlet_form(F[i], J[i]) == 3) {
             blocks += comb_chunks(F[i], 1);
-            if (F[i] <= kClusterMaxF) ++clusters;
+            if (F[i] <= kClusterMaxF) shapes.push_back({F[i], J[i] - 1});
         }
     if (blocks == 0 || blocks >= 2LL * n_sms) return 0;
     const int rows = 2 * blocks >= 2LL * n_sms ? kStarletRows8 : kStarletRows4;
-    return rows | (clusters > 0 && 3 * clusters * kClusterBlocks <= 2LL * n_sms ? kStarletClusterBit : 0);
+    return rows | (starlet_clusters(shapes, n_sms) ? kStarletClusterBit : 0);
 }
 
 int launch_starlet(const FieldDev *fields, int n_fields, int Fmax, int forms, const ChunkItem *chunks,

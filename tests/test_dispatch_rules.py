@@ -46,15 +46,17 @@ def test_the_form_autotuner_times_the_tiles_of_full_batches():
     assert {rows(_ints([E]), _ints([64]), 1, 152, 1) for E in (1, 4, 16)} == {64}
 
 
-def test_clusters_only_where_they_run_at_once():
-    """Starlet clusters: grids up to 256 pixels, in tables whose clusters leave a third of the SMs free."""
+def test_clusters_only_where_they_do_not_queue():
+    """Starlet clusters: grids up to 256 pixels, in tables whose clusters do not wait long for one another."""
     bits, cluster = _rule("_ZN2sr22starlet_comb_rows_bitsEPKiS1_ii"), 128
 
-    def has(*F):
-        return bool(bits(_ints(F), _ints([4] * len(F)), len(F), 152) & cluster)
+    def has(F, J):
+        return bool(bits(_ints(F), _ints(J), len(F), 152) & cluster)
 
-    assert has(64) and has(*[128] * 12) and has(256) and has(420, 128)
-    assert not has(*[64] * 16) and not has(*[256] * 16) and not has(420) and not has(600, 300)
+    assert has([64], [4]) and has([128] * 12, [4] * 12) and has([256], [4]) and has([420, 128], [5, 4])
+    assert has([64, 96, 128] * 8, [4, 5, 6] * 8)
+    assert not has([64] * 16, [4] * 16) and not has([128] * 32, [6] * 32) and not has([64, 96] * 19, [4, 6] * 19)
+    assert not has([420], [5]) and not has([600, 300], [5, 5])
 
 
 def test_shift_gradient_threads_follow_the_grid(tmp_path):
