@@ -184,7 +184,7 @@ struct BranchStreams {
     enum { kPrior, kPts, kSrc, kStep, kCount };
     std::mutex m;
     cudaStream_t s[kCount][2] = {};
-    std::atomic<unsigned> turn[kCount] = {};
+    unsigned turn[kCount] = {};
     ~BranchStreams() {
         for (auto &pair : s)
             for (cudaStream_t st : pair)
@@ -192,11 +192,25 @@ struct BranchStreams {
     }
     sr_status open(int k) {
         std::lock_guard<std::mutex> lock(m);
-        for (cudaStream_t &st : s[k])
-            if (!st) SR_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+        if (!s[k][0]) SR_CUDA(cudaStreamCreateWithFlags(&s[k][0], cudaStreamNonBlocking));
         return SR_OK;
     }
-    cudaStream_t next(int k) { return s[k][turn[k].fetch_add(1, std::memory_order_relaxed) & 1]; }
+    // The branch's next stream for a fork from `st`. The second one is opened when its turn first comes (a first
+    // evaluation does not pay for it), not inside a capture.
+    cudaStream_t next(int k, cudaStream_t st) {
+        std::lock_guard<std::mutex> lock(m);
+        const unsigned i = turn[k]++ & 1;
+        if (!s[k][i]) {
+            cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+                cudaStreamCreateWithFlags(&s[k][i], cudaStreamNonBlocking) != cudaSuccess) {
+                cudaGetLastError();
+                s[k][i] = nullptr;
+                return s[k][0];
+            }
+        }
+        return s[k][i];
+    }
 };
 
 static std::mutex g_branch_mutex;
@@ -256,7 +270,7 @@ struct Branch {
     // (or when the fork fails: the order is then kept)
     cudaStream_t fork(cudaStream_t st) {
         if (!set) return st;
-        cudaStream_t stream = set->next(kind);
+        cudaStream_t stream = set->next(kind, st);
         if (cudaEventRecord(forked, st) != cudaSuccess || cudaStreamWaitEvent(stream, forked, 0) != cudaSuccess) {
             cudaGetLastError();
             return st;
