@@ -122,7 +122,8 @@ extern "C" sr_status sr_loss_and_grad_noalloc(const sr_problem_desc *desc, const
     SR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     SR_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
 
-    // geometry of the folded kernels and of the output tiles (the same rules as a created problem)
+    // geometry of the folded kernels (as a created problem's) and of the output tiles: 64 rows, one partial sum
+    // each, so that the scratch does not depend on the number of epochs per SM
     const int o = K / 2, t_lo = -o - f + 1, t_hi = K - 1 - o;
     const int tau_lo = t_lo >= 0 ? (t_lo + f - 1) / f : -((-t_lo) / f);
     const int tau_hi = (t_hi + f - 1) >= 0 ? (t_hi + f - 1) / f : -((-(t_hi + f - 1) + f - 1) / f);
