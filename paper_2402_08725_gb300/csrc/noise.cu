@@ -505,7 +505,7 @@ noise_setup_kernel(const float *__restrict__ sigma, const float *__restrict__ s1
 // 1.8: 1.0 / 0.8, 2.8: 1.0 / 0.9, 5.2: 1.0 / 1.3; K = 21, 4.0: 2.3 / 2.0, 5.2: 2.2 / 2.2; K = 33, 5.2: 3.6 / 2.1, 10:
 // 3.6 / 4.2; K = 64, 9.2: 2.6 / 1.4 (the second plane equal there), 18: 2.5 / 2.7.  Hence K / 8, at least
 // 2.5: an even grid has 1.8 (a quarter of the PSF at its corners), a 300-epoch quasar field 3.2.
-constexpr int kLevelBox = 6, kLevelBlocks = 128;
+constexpr int kLevelBox = 6, kLevelBlocks = 152;
 constexpr float kLevelRange = 1e12f;  // 1 / sigma_eff and the PSF's norm within 1e-12 .. 1e12: no overflow
 struct LevelPart {
     float least, most;  // level^2, isig
@@ -520,13 +520,14 @@ __device__ __noinline__ void noise_level(const float *__restrict__ isig, const f
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = K / 2;
     const int cy = peak->qy - kLevelBox, cx = peak->qx - kLevelBox;
     LevelPart p{INFINITY, 0.f, 0.0};
-    for (int u = b * 256 + threadIdx.x; u < F * F; u += nb * 256) {
-        const int y = u / F, x = u - y * F;
+    // four lanes a pixel, each a quarter of the box's rows
+    for (int w = b * 256 + (int)threadIdx.x - lane; w < 4 * F * F; w += nb * 256) {
+        const int u = (w + lane) >> 2, y = u / F, x = u - y * F;
         float lv = 0.f;
-#pragma unroll 2
-        for (int a = 0; a <= 2 * kLevelBox; ++a) {
-            const int qy = cy + a, gy = y + qy - o;
-            if (qy < 0 || qy >= K || gy < 0 || gy >= F) continue;
+#pragma unroll
+        for (int a0 = 0; a0 <= 2 * kLevelBox; a0 += 4) {
+            const int a = a0 + (lane & 3), qy = cy + a, gy = y + qy - o;
+            if (a > 2 * kLevelBox || u >= F * F || qy < 0 || qy >= K || gy < 0 || gy >= F) continue;
             float v[2 * kLevelBox + 1];
 #pragma unroll
             for (int c = 0; c <= 2 * kLevelBox; ++c) {  // a row's loads together
@@ -537,10 +538,14 @@ __device__ __noinline__ void noise_level(const float *__restrict__ isig, const f
 #pragma unroll
             for (int c = 0; c <= 2 * kLevelBox; ++c) lv = fmaf(v[c], v[c], lv);
         }
-        const float i = isig[u];
-        p.least = fminf(p.least, lv);
-        p.most = fmaxf(p.most, i);
-        p.power += (double)i * (double)i;
+        lv += __shfl_xor_sync(0xffffffffu, lv, 1);
+        lv += __shfl_xor_sync(0xffffffffu, lv, 2);
+        if (u < F * F && (lane & 3) == 0) {
+            const float i = isig[u];
+            p.least = fminf(p.least, lv);
+            p.most = fmaxf(p.most, i);
+            p.power += (double)i * (double)i;
+        }
     }
     auto join = [](LevelPart a, LevelPart b) { return LevelPart{fminf(a.least, b.least), fmaxf(a.most, b.most), a.power + b.power}; };
     auto warp_join = [&](LevelPart a) {
@@ -765,7 +770,7 @@ extern "C" sr_status sr_noise_weights(int N, int f, int K, int J, int E, const f
     noise_setup_kernel<<<n_isig + spec.L + (use_fft ? 1 : 0), 32 * kIsigWarps, 0, st>>>(sigma_dev, s1_dev, N, f, E, K,
                                                                                         n_isig, isig, flag, spec, peak);
     ++launches;
-    const int n_level = (int)std::min<long long>((FF + 255) / 256, kLevelBlocks);
+    const int n_level = (int)std::min<long long>((4 * FF + 255) / 256, kLevelBlocks);
     // The transforms' first batch runs before the host knows whether they are to be used: asking first would
     // leave the GPU idle for the answer (a call of 400 us took 445).
     bool fft_now = use_fft;
