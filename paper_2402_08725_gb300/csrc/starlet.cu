@@ -12,8 +12,8 @@
 // and two T planes (J, J+1) used alternately; T_0 ends in plane J.
 //
 // Four ways to run, chosen per field (starlet_form) and table:
-//  * clusters (grids up to 256 pixels in tables of a few fields): all levels of a field in one launch, on
-//    a cluster of 8 blocks that take the comb bands below, with a cluster barrier between levels instead
+//  * clusters (grids up to 256 pixels, where starlet_clusters finds that faster): all levels of a field in
+//    one launch, on a cluster of 8 blocks that take the comb bands below, with a cluster barrier between levels instead
 //    of a launch (see starlet_cluster_kernel).
 //  * comb bands (most fields): the rows rho, rho + s, rho + 2 s, ... of level j (step s = 2^j)
 //    are one column tap apart, so a block taking 16 consecutive rows of one such comb stages
